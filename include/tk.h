@@ -103,15 +103,17 @@ int tk_row_align(int m, int64_t n, int64_t off, int64_t *row_off_host);
  * X: n x d row-major FP64 (device).  K: N entries of storage_dtype (device,
  * caller-allocated with tk_packed_bytes bytes).  Accumulation is FP64 for
  * TK_F64 storage and FP32 otherwise; TK_BF16 rounds the FP32 result to
- * nearest-even.  `degree` is used by TK_FEAT_POLY only.  No workspace. */
+ * nearest-even.  `degree` is used by TK_FEAT_POLY only.  No workspace: the
+ * tensor-core build takes stream-ordered memory for its operand images
+ * (tk_build_workspace_size bytes; without it the SIMT build runs). */
 int tk_build_packed(int m, int64_t n, int64_t d, const double *X, int feat,
                     int degree, int storage_dtype, void *K, void *stream);
 
-/* Which kernel builds FP32 / BF16 storage: 0 (default) and -1 = the SIMT
- * build, 1 = the tensor-core build (tcgen05.mma kind::tf32 with the 3-term
- * split, a warp-specialised pipeline over 128 x 128 tiles of each triangle),
- * which is correct but measured slower on GB300.  FP64 storage always takes
- * the SIMT build.  Process-wide. */
+/* Which kernel builds FP32 / BF16 storage: 0 (default) = the tensor-core build
+ * (tcgen05.mma kind::f16 over three-part BF16 splits of the operands) for orders
+ * m >= 3 beyond the smallest sizes (but not for the exponential map into FP32), 1 =
+ * for every build of m >= 3, -1 = the SIMT build.  FP64 storage is built on the
+ * FP64 units.  Process-wide. */
 int tk_build_set_config(int tensor_cores);
 
 /* Status of the tensor-core builds issued so far on the current device:
@@ -119,8 +121,9 @@ int tk_build_set_config(int tensor_cores);
  * to be trusted), else TK_OK; reading clears it.  Synchronises `stream`. */
 int tk_build_status(void *stream);
 
-/* 1 if a build of d features into storage_dtype takes the tensor-core build
- * under the current configuration on the current device, else 0. */
+/* 1 if builds of d features into storage_dtype take the tensor-core build
+ * (beyond the smallest sizes) under the current configuration on the current
+ * device, else 0. */
 int tk_build_path(int64_t d, int storage_dtype);
 
 /* Same for the offsets [off_lo, off_hi) only: K_range[o - off_lo] = K[o].
@@ -128,6 +131,18 @@ int tk_build_path(int64_t d, int storage_dtype);
 int tk_build_packed_range(int m, int64_t n, int64_t d, const double *X, int feat,
                           int degree, int storage_dtype, int64_t off_lo,
                           int64_t off_hi, void *K_range, void *stream);
+
+/* The same with the caller's workspace (device memory, no alignment needed):
+ * tk_build_workspace_size bytes let the tensor-core build make its operand
+ * images at once (or in panels of 2 GB); with less it works in smaller panels,
+ * with the same results, down to one tile of each operand (TK_ENOMEM below).
+ * work == NULL: as tk_build_packed_range.  The size is 0 where no workspace is
+ * used (FP64 storage, m = 2, the SIMT build). */
+size_t tk_build_workspace_size(int m, int64_t n, int64_t d, int storage_dtype);
+int tk_build_packed_work(int m, int64_t n, int64_t d, const double *X, int feat,
+                         int degree, int storage_dtype, int64_t off_lo,
+                         int64_t off_hi, void *K_range, void *work,
+                         size_t work_bytes, void *stream);
 
 /* ------------------------------------------------------------ contraction */
 

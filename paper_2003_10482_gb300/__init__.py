@@ -69,6 +69,8 @@ def _declare(L):
         "tk_row_align": (i32, [i32, i64, i64, P]),
         "tk_build_packed": (i32, [i32, i64, i64, P, i32, i32, i32, P, P]),
         "tk_build_packed_range": (i32, [i32, i64, i64, P, i32, i32, i32, i64, i64, P, P]),
+        "tk_build_workspace_size": (sz, [i32, i64, i64, i32]),
+        "tk_build_packed_work": (i32, [i32, i64, i64, P, i32, i32, i32, i64, i64, P, P, sz, P]),
         "tk_contract_workspace_size": (sz, [i32, i64, i64]),
         "tk_contract": (i32, [i32, i64, i32, P, i64, i32, P, i32, P, P, P, P, sz, P]),
         "tk_contract_range": (i32, [i32, i64, i32, P, i64, i64, i64, i32, P, i32, P, P, P, P, sz, P]),
@@ -302,8 +304,8 @@ def tk_umma_probe(A: torch.Tensor, B: torch.Tensor, split: bool = False, stream=
 
 
 def tk_build_set_config(tensor_cores: int = 0) -> None:
-    """Which kernel builds FP32 / BF16 storage: 0 = tensor cores where they pay,
-    1 = always the tensor-core build, -1 = always the SIMT build."""
+    """Which kernel builds FP32 / BF16 storage: 0 = the tensor-core build where it
+    pays, 1 = always (orders m >= 3), -1 = the SIMT build."""
     _check(lib().tk_build_set_config(int(tensor_cores)))
 
 
@@ -337,11 +339,19 @@ def tk_build_packed(X: torch.Tensor, m: int, storage="f32", feat="linear", degre
         K = torch.empty(hi - lo, dtype=_TORCH[code], device=X.device)
     assert K.numel() >= hi - lo and K.dtype == _TORCH[code]
     f = _FEAT[feat] if isinstance(feat, str) else int(feat)
-    if off_lo is None and off_hi is None:
-        _check(lib().tk_build_packed(m, n, d, _p(X), f, degree, code, _p(K), _stream(stream)))
-    else:
-        _check(lib().tk_build_packed_range(m, n, d, _p(X), f, degree, code, lo, hi, _p(K),
-                                           _stream(stream)))
+    # operand images of the tensor-core build, from PyTorch's pool (on another
+    # stream than the current one the library takes stream-ordered memory itself)
+    work = None
+    need = int(lib().tk_build_workspace_size(m, n, d, code)) if stream is None and f != TK_FEAT_EXP else 0
+    for size in (need, need // 4, need // 16) if need else ():
+        try:
+            work = torch.empty(size, dtype=torch.uint8, device=X.device)
+            break
+        except torch.cuda.OutOfMemoryError:
+            continue  # smaller panels, the same results
+    rc = lib().tk_build_packed_work(m, n, d, _p(X), f, degree, code, lo, hi, _p(K), _p(work),
+                                    0 if work is None else work.numel(), _stream(stream))
+    _check(rc)
     return K
 
 

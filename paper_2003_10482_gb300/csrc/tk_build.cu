@@ -1,8 +1,19 @@
 // Packed build of the order-m tensor kernel (Section 4), stored in the
-// sorted-tuple order of Section 5.
+// sorted-tuple order of Section 5, on the FP32 and FP64 units; tk_build_tc.cu
+// holds the tensor-core build, which takes FP32 / BF16 storage beyond the
+// smallest sizes (build_uses_tc).
 //
-// For a triangle Q = (i_1..i_{m-2}) with last value b, the entries (Q, c, d),
-// b <= c <= d < n, form the upper triangle of the weighted Gram matrix
+// build_pairs_f64 (FP64 storage, m >= 3) is the matrix product prefixes x pairs
+// of tk_build_tc.cu on the FP64 units.  GB300 does two FP64 multiply-adds per
+// cycle and SM, so that pipe is all that counts: what helps is to form no
+// products for padding.  m = 4, n = 120, d = 32: 2.44 ms with build_kernel's
+// 64 x 64 tiles per triangle (four fifths of their products outside the
+// triangles), 0.61 ms here, 0.95 of the units' measured 1.06 TFLOP/s.
+//
+// build_kernel (m = 2; FP32 storage under the exponential map; FP32 / BF16 storage of
+// small arrays, or where the tensor cores are switched off): for a triangle Q = (i_1..i_{m-2}) with last value b,
+// the entries (Q, c, d), b <= c <= d < n, form the upper triangle of the
+// weighted Gram matrix
 //   G^Q = X_{[b:n]} diag(w_Q) X_{[b:n]}^T,   w_Q[k] = prod_{q in Q} x_{q,k},
 // i.e. K_{Qcd} = sum_k w_Q[k] x_{c,k} x_{d,k}.  Each block computes one 64 x 64
 // tile of one such triangle as a small GEMM (16 x 16 threads, 4 x 4 outputs
@@ -14,11 +25,9 @@
 // T(n-b) = nb(nb+1)/2 tile pairs (nb = ceil((n-b)/64)).  A persistent grid
 // strides over the tasks; each block builds the per-b prefix table of task
 // counts in shared memory once.
-#include <cuda_bf16.h>
-
 #include <algorithm>
 
-#include "tk_internal.h"
+#include "tk_build.cuh"
 
 namespace tk {
 
@@ -41,32 +50,6 @@ __device__ __forceinline__ int tiles_for(int L) {
 
 __device__ __forceinline__ float fmx(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmx(double a, double b, double c) { return __fma_rn(a, b, c); }
-
-template <typename CT>
-__device__ __forceinline__ CT feat_apply(CT v, int feat, int degree) {
-  if (feat == TK_FEAT_POLY) {
-    CT r = CT(1);
-    for (int i = 0; i < degree; ++i) r *= v;
-    return r;
-  }
-  if (feat == TK_FEAT_EXP) return exp(v);
-  return v;
-}
-
-template <typename ST, typename CT>
-__device__ __forceinline__ void store_entry(void *K, int64_t idx, CT v);
-template <>
-__device__ __forceinline__ void store_entry<double, double>(void *K, int64_t idx, double v) {
-  reinterpret_cast<double *>(K)[idx] = v;
-}
-template <>
-__device__ __forceinline__ void store_entry<float, float>(void *K, int64_t idx, float v) {
-  reinterpret_cast<float *>(K)[idx] = v;
-}
-template <>
-__device__ __forceinline__ void store_entry<__nv_bfloat16, float>(void *K, int64_t idx, float v) {
-  reinterpret_cast<__nv_bfloat16 *>(K)[idx] = __float2bfloat16_rn(v);
-}
 
 template <typename ST, typename CT>
 __global__ void __launch_bounds__(256) build_kernel(BParams p) {
@@ -189,6 +172,117 @@ __global__ void __launch_bounds__(256) build_kernel(BParams p) {
   }
 }
 
+// The FP64 build (m >= 3): the matrix product of tk_build_tc.cu, prefixes
+// ordered by their last value against pairs (c, d), on the FP64 units.  A block
+// computes one TM x TM tile, 16 x 16 threads with TM/16 x TM/16 outputs each at
+// a stride of 16 (consecutive threads on consecutive entries), 16 features per
+// stage; blockIdx.x is the column tile, blockIdx.y strides over the row tiles,
+// and tiles before the row tile's first pair end at once.
+template <int TM>
+__global__ void __launch_bounds__(256) build_pairs_f64(BParams p, BuildShape s) {
+  constexpr int R = TM / 16;
+  __shared__ double Ws[kKT][TM + 1], Ps[kKT][TM + 1];
+  __shared__ int64_t obase[TM];
+  __shared__ int sb[TM];
+  __shared__ uint16_t tw[TM][kMaxOrder], tp[TM][2];
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const int m = p.m, n = p.n, d = p.d;
+  const int64_t p0 = (int64_t)blockIdx.x * TM;
+  const int64_t nrt = (s.rows + TM - 1) / TM;
+  for (int64_t rt = blockIdx.y; rt < nrt; rt += gridDim.y) {
+    // rows are ordered by b: the first row's is the smallest
+    if (build_first_pair(n, build_row_last(s, rt * TM)) >= p0 + TM) return;
+    __syncthreads();
+    if (tid < TM) {
+      const int64_t row = rt * TM + tid;
+      int32_t t[kMaxOrder];
+      sb[tid] = 0x7fffffff;
+      obase[tid] = 0;
+      for (int j = 0; j < m - 2; ++j) tw[tid][j] = 0;
+      if (row < s.rows) {
+        const int b = build_row_tuple(s, row, t);
+        t[m - 2] = b;
+        t[m - 1] = b;
+        sb[tid] = build_first_pair(n, b);
+        obase[tid] = rank(m, n, t) - sb[tid];
+        for (int j = 0; j < m - 2; ++j) tw[tid][j] = (uint16_t)t[j];
+      }
+    } else if (tid < 2 * TM) {
+      const int i = tid - TM;
+      int32_t t[2] = {0, 0};
+      if (p0 + i < s.pairs) unrank(2, n, p0 + i, t);
+      tp[i][0] = (uint16_t)t[0];
+      tp[i][1] = (uint16_t)t[1];
+    }
+    double acc[R][R];
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+      for (int j = 0; j < R; ++j) acc[i][j] = 0.0;
+    for (int k0 = 0; k0 < d; k0 += kKT) {
+      __syncthreads();
+      const int k = k0 + tx;
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const int r = ty + 16 * i;
+        double w = 0.0, q = 0.0;
+        if (k < d) {
+          w = p.X[(int64_t)tw[r][0] * d + k];
+          for (int j = 1; j < m - 2; ++j) w *= p.X[(int64_t)tw[r][j] * d + k];
+          q = p.X[(int64_t)tp[r][0] * d + k] * p.X[(int64_t)tp[r][1] * d + k];
+        }
+        Ws[tx][r] = w;
+        Ps[tx][r] = q;
+      }
+      __syncthreads();
+      const int nk = min(kKT, d - k0);
+#pragma unroll 4
+      for (int kk = 0; kk < nk; ++kk) {
+        double a[R], b[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          a[i] = Ws[kk][ty + 16 * i];
+          b[i] = Ps[kk][tx + 16 * i];
+        }
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+          for (int j = 0; j < R; ++j) acc[i][j] = fmx(a[i], b[j], acc[i][j]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int r = ty + 16 * i;
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        const int64_t q = p0 + tx + 16 * j, off = obase[r] + q;
+        if (q < sb[r] || q >= s.pairs || off < p.off_lo || off >= p.off_hi) continue;
+        store_entry<double, double>(p.K, off - p.off_lo, feat_apply(acc[i][j], p.feat, p.degree));
+      }
+    }
+  }
+}
+
+static int launch_pairs_f64(const BParams &bp, cudaStream_t st) {
+  DevInfo di;
+  int rc = dev_info(&di);
+  if (rc != TK_OK) return rc;
+  int32_t t[16];
+  unrank(bp.m, bp.n, bp.off_lo, t);
+  const int i_lo = t[0];
+  unrank(bp.m, bp.n, bp.off_hi - 1, t);
+  const BuildShape s = build_shape(bp.m, bp.n, i_lo, t[0]);
+  auto tiles = [&](int tm) { return ((s.rows + tm - 1) / tm) * ((s.pairs + tm - 1) / tm); };
+  // about a third of the (row tile, column tile) grid lies past its row tile's
+  // first pair: 64-wide tiles while they still fill the SMs several times
+  const int tm = tiles(64) >= (int64_t)24 * di.sms ? 64 : 32;
+  const dim3 grid((unsigned)((s.pairs + tm - 1) / tm), (unsigned)std::min<int64_t>((s.rows + tm - 1) / tm, 32768));
+  if (tm == 64) build_pairs_f64<64><<<grid, 256, 0, st>>>(bp, s);
+  else build_pairs_f64<32><<<grid, 256, 0, st>>>(bp, s);
+  TK_CUDA_CHECK(cudaGetLastError());
+  return TK_OK;
+}
+
 template <typename ST, typename CT>
 static int launch_build(const BParams &bp, cudaStream_t st) {
   DevInfo di;
@@ -215,30 +309,69 @@ extern "C" int tk_build_set_config(int tensor_cores) {
 
 extern "C" int tk_build_status(void *stream) { return build_tc_status(reinterpret_cast<cudaStream_t>(stream)); }
 
-static bool build_takes_tc(int64_t d, int storage) {
-  // the tensor-core build is opt-in: on GB300 it measured slower than the SIMT
-  // build (m = 4: n = 200, d = 20,000: 501 vs 443 ms; n = 400, d = 100: 56 vs
-  // 29 ms), bound by its operand-building warps rather than the tensor cores
-  (void)d;
-  if (storage == TK_F64 || g_build_tc_mode <= 0) return false;
+// tasks of build_kernel: (triangle, tile pair)
+static int64_t build_tasks(int m, int64_t n) {
+  auto tiles = [](int64_t L) {
+    const int64_t nb = (L + kTM - 1) / kTM;
+    return nb * (nb + 1) / 2;
+  };
+  if (m == 2) return tiles(n);
+  int64_t total = 0;
+  for (int64_t b = 0; b < n; ++b) total += multiset(b + 1, m - 3) * tiles(n - b);
+  return total;
+}
+
+// FP32 / BF16 storage goes to the tensor cores from kMinTcStages 16-feature
+// stages of build_kernel on: that kernel takes some 25 us + 13 ns per stage
+// (m = 4: n = 40, d = 10, 820 stages 37 us; n = 60, d = 30, 3660 stages 70 us), the
+// tensor-core build's three launches 45-50 us at those sizes.
+constexpr int64_t kMinTcStages = 1500;
+static bool build_takes_tc(int storage) {
+  if (storage == TK_F64 || g_build_tc_mode < 0) return false;
   int dev = 0, major = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return false;
   return major == 10;
 }
 
-extern "C" int tk_build_path(int64_t d, int storage) { return build_takes_tc(d, storage) ? 1 : 0; }
+extern "C" int tk_build_path(int64_t d, int storage) {
+  (void)d;
+  return build_takes_tc(storage) ? 1 : 0;
+}
 
-extern "C" int tk_build_packed_range(int m, int64_t n, int64_t d, const double *X, int feat, int degree,
-                                     int storage, int64_t off_lo, int64_t off_hi, void *K, void *stream) {
+static bool build_uses_tc(int m, int64_t n, int64_t d, int feat, int storage) {
+  if (m < 3 || !build_takes_tc(storage)) return false;
+  if (g_build_tc_mode > 0) return true;
+  // exp(s) turns the rounding of s, some 1e-7 |s|, into a relative error of the
+  // entry (2e-5 at the exponents FP32 can hold): FP32 storage keeps the sums,
+  // and so the entries, of the multiply-add build there
+  if (feat == TK_FEAT_EXP && storage == TK_F32) return false;
+  return build_tasks(m, n) * ((d + kKT - 1) / kKT) > kMinTcStages;
+}
+
+static int check_build(int m, int64_t n, int64_t d, int feat, int degree, int storage) {
   if (m < 2 || m > TK_MAX_ORDER) return fail(TK_EINVAL, "order m=%d outside [2, %d]", m, TK_MAX_ORDER);
   if (n < 1 || d < 1) return fail(TK_EINVAL, "n and d must be >= 1");
   if (n > TK_MAX_POINTS) return fail(TK_EUNSUPPORTED, "n=%lld exceeds %d", (long long)n, TK_MAX_POINTS);
   if (storage < TK_F64 || storage > TK_BF16) return fail(TK_EINVAL, "bad storage dtype %d", storage);
   if (feat < TK_FEAT_LINEAR || feat > TK_FEAT_EXP) return fail(TK_EINVAL, "bad feature map %d", feat);
   if (feat == TK_FEAT_POLY && degree < 1) return fail(TK_EINVAL, "polynomial degree must be >= 1");
+  if (tk_packed_size(m, n) < 0) return fail(TK_EOVERFLOW, "C(n+m-1, m) overflows");
+  return TK_OK;
+}
+
+extern "C" size_t tk_build_workspace_size(int m, int64_t n, int64_t d, int storage) {
+  if (check_build(m, n, d, TK_FEAT_LINEAR, 1, storage) != TK_OK) return 0;
+  if (!build_uses_tc(m, n, d, TK_FEAT_LINEAR, storage)) return 0;
+  return build_tc_workspace_bytes(m, (int)n, (int)d);
+}
+
+extern "C" int tk_build_packed_work(int m, int64_t n, int64_t d, const double *X, int feat, int degree, int storage,
+                                    int64_t off_lo, int64_t off_hi, void *K, void *work, size_t work_bytes,
+                                    void *stream) {
+  int rc = check_build(m, n, d, feat, degree, storage);
+  if (rc != TK_OK) return rc;
   const int64_t N = tk_packed_size(m, n);
-  if (N < 0) return fail(TK_EOVERFLOW, "C(n+m-1, m) overflows");
   if (off_lo < 0 || off_hi > N || off_lo > off_hi) return fail(TK_EINVAL, "range outside [0, N]");
   if (off_hi == off_lo) return TK_OK;
   if (!X || !K) return fail(TK_EINVAL, "NULL X or K");
@@ -252,25 +385,37 @@ extern "C" int tk_build_packed_range(int m, int64_t n, int64_t d, const double *
   bp.K = K;
   bp.off_lo = off_lo;
   bp.off_hi = off_hi;
-  int64_t total = 0;
-  if (m == 2) {
-    const int nb = (int)((n + kTM - 1) / kTM);
-    total = (int64_t)nb * (nb + 1) / 2;
-  } else {
-    for (int64_t b = 0; b < n; ++b) {
-      const int64_t L = n - b, nb = (L + kTM - 1) / kTM;
-      total += multiset(b + 1, m - 3) * (nb * (nb + 1) / 2);
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (build_uses_tc(m, n, d, feat, storage)) {
+    // without a workspace of the caller's: stream-ordered memory for the call
+    void *own = nullptr;
+    if (!work) {
+      work_bytes = build_tc_workspace_bytes(m, (int)n, (int)d);
+      if (cudaMallocAsync(&own, work_bytes, st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        own = nullptr;
+      }
+      work = own;
+    }
+    if (work) {
+      rc = build_tc(m, (int)n, (int)d, X, feat, degree, storage, off_lo, off_hi, K, work, work_bytes, st);
+      if (own) {
+        const cudaError_t e = cudaFreeAsync(own, st);
+        if (rc == TK_OK && e != cudaSuccess) return cuda_fail(e, "cudaFreeAsync");
+      }
+      if (rc != TK_EUNSUPPORTED) return rc;
     }
   }
-  bp.total_tasks = total;
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (build_takes_tc(d, storage)) {
-    const int rc = build_tc(m, (int)n, (int)d, X, feat, degree, storage, off_lo, off_hi, K, st);
-    if (rc != TK_EUNSUPPORTED) return rc;
-  }
+  if (m >= 3 && storage == TK_F64) return launch_pairs_f64(bp, st);
+  bp.total_tasks = build_tasks(m, n);
   if (storage == TK_F64) return launch_build<double, double>(bp, st);
   if (storage == TK_F32) return launch_build<float, float>(bp, st);
   return launch_build<__nv_bfloat16, float>(bp, st);
+}
+
+extern "C" int tk_build_packed_range(int m, int64_t n, int64_t d, const double *X, int feat, int degree,
+                                     int storage, int64_t off_lo, int64_t off_hi, void *K, void *stream) {
+  return tk_build_packed_work(m, n, d, X, feat, degree, storage, off_lo, off_hi, K, nullptr, 0, stream);
 }
 
 extern "C" int tk_build_packed(int m, int64_t n, int64_t d, const double *X, int feat, int degree, int storage,

@@ -1,0 +1,83 @@
+// Shared by the packed builds (tk_build.cu, tk_build_tc.cu): the order of the
+// prefix rows of the build product and the epilogue of an entry.
+#pragma once
+#include <cuda_bf16.h>
+
+#include "tk_internal.h"
+
+namespace tk {
+
+// The rows of the build product: the prefixes Q = (i_1..i_{m-2}) (m >= 3) with
+// i_lo <= i_1 <= i_hi, ordered by their last value b, then lexicographically;
+// its columns: the pairs (c, d), c <= d, in lexicographic order.
+struct BuildShape {
+  int m, n;
+  int i_lo, i_hi;
+  int64_t rows, pairs;
+};
+
+// rows whose last value lies below b: the sorted (m-2)-tuples over [i_lo, b)
+// without those over (i_hi, b)
+TK_HD int64_t build_rows_below(const BuildShape &s, int b) {
+  return multiset(b - s.i_lo, s.m - 2) - multiset(b - 1 - s.i_hi, s.m - 2);
+}
+
+inline BuildShape build_shape(int m, int n, int i_lo, int i_hi) {
+  BuildShape s{m, n, i_lo, i_hi, 0, (int64_t)n * (n + 1) / 2};
+  s.rows = build_rows_below(s, n);
+  return s;
+}
+
+// last value of row `row`: the largest b with build_rows_below(b) <= row
+TK_HD int build_row_last(const BuildShape &s, int64_t row) {
+  int lo = s.i_lo, hi = s.n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (build_rows_below(s, mid) <= row) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
+// the prefix of row `row` into t[0..m-3]; returns its last value
+TK_HD int build_row_tuple(const BuildShape &s, int64_t row, int32_t *t) {
+  const int b = build_row_last(s, row);
+  if (s.m > 3) {
+    // within b the (m-3)-tuples over [0, b] in lexicographic order, from the
+    // first one whose first value is i_lo on
+    const int64_t skip = multiset(b + 1, s.m - 3) - multiset(b + 1 - s.i_lo, s.m - 3);
+    unrank(s.m - 3, b + 1, skip + row - build_rows_below(s, b), t);
+  }
+  t[s.m - 3] = b;
+  return b;
+}
+
+// index of the pair (b, b)
+TK_HD int build_first_pair(int n, int b) { return (int)((int64_t)b * (2 * n - b + 1) / 2); }
+
+template <typename CT>
+__device__ __forceinline__ CT feat_apply(CT v, int feat, int degree) {
+  if (feat == TK_FEAT_POLY) {
+    CT r = CT(1);
+    for (int i = 0; i < degree; ++i) r *= v;
+    return r;
+  }
+  if (feat == TK_FEAT_EXP) return exp(v);
+  return v;
+}
+
+template <typename ST, typename CT>
+__device__ __forceinline__ void store_entry(void *K, int64_t idx, CT v);
+template <>
+__device__ __forceinline__ void store_entry<double, double>(void *K, int64_t idx, double v) {
+  reinterpret_cast<double *>(K)[idx] = v;
+}
+template <>
+__device__ __forceinline__ void store_entry<float, float>(void *K, int64_t idx, float v) {
+  reinterpret_cast<float *>(K)[idx] = v;
+}
+template <>
+__device__ __forceinline__ void store_entry<__nv_bfloat16, float>(void *K, int64_t idx, float v) {
+  reinterpret_cast<__nv_bfloat16 *>(K)[idx] = __float2bfloat16_rn(v);
+}
+
+}  // namespace tk

@@ -1,383 +1,599 @@
-// Packed build on the 5th-generation tensor cores (FP32 and BF16 storage).
+// Packed build of FP32 / BF16 storage on the 5th-generation tensor cores
+// (Section 4 tensor kernel, stored in the order of Section 5).
 //
-// What is computed is the build of tk_build.cu (Section 4 tensor kernel,
-// Section 5 storage): for a triangle Q with last value b the entries
-// (Q, c, d), b <= c <= d < n, are the upper triangle of the weighted Gram
-// matrix G^Q = X_{[b:n]} diag(w_Q) X_{[b:n]}^T, w_Q[k] = prod_{q in Q} x_{q,k},
-// passed through the feature map.
+// The packed array as a matrix product.  Split a sorted tuple into its prefix
+// Q = (i_1..i_{m-2}) with last value b and the pair (c, d), b <= c <= d.  The
+// entries of one Q are contiguous in the packed array and run over the pairs
+// (c, d) in lexicographic order from s(b) = b(2n-b+1)/2 on, so
+//   K[base(Q) + p - s(b)] = sum_k W[Q][k] P[p][k],
+//   W[Q][k] = prod_{q in Q} x_{q,k},  P[p][k] = x_{c,k} x_{d,k},
+// is one product of the prefixes' rows with the pairs' rows, whose output
+// rows are contiguous.  With the prefixes ordered by b only the tiles that the
+// line p = s(b) crosses compute entries nobody needs (at m = 4, n = 400 under
+// 2 % of them), whatever the size of the single triangles.
 //
-// GB300 mapping.  The triangles with last value b (multiset(b+1, m-3) of them)
-// share their rows and columns [b, n), L = n - b.  A task is one MMA tile of
-// 128 rows: for L <= 128 the rows of floor(128/L) consecutive such triangles
-// stacked (columns [b, n)); for L > 128 one triangle's 128-row block c in
-// [b + 128 rt, ...) against the 128-column block d in [b + 128 ct, ...),
-// ct >= rt.  Tasks are enumerated per b and strided over a persistent grid of
-// one block per SM.  The block is a warp-specialised pipeline connected by
-// mbarriers:
-//   * warps 4-11 build, per 32-feature chunk, both operands from X in FP64 --
-//     A[r][k] = x_{c_r,k} prod_{q in Q_r} x_{q,k} for row r's triangle Q_r and
-//     row c_r, B[j][k] = x_{d_j,k} -- with each triangle's weight row formed
-//     once per chunk (rounded to FP32), lanes along the features (coalesced
-//     loads, all of a warp's rows issued before use), round them to FP32,
-//     split them into TF32 hi and lo and store them in the K-major
-//     128-byte-swizzled layout of one of 3 ring stages;
-//   * one thread of warp 12 issues 4 k-steps of tcgen05.mma kind::tf32
-//     (M = 128 rows, N = the tile's columns, K = 8): hi.hi into one tensor-
-//     memory accumulator, hi.lo + lo.hi into a second (the large products
-//     summed apart from the small ones), two such pairs alternating between
-//     tasks;
-//   * warps 0-3 (thread i <-> tensor-memory lane i <-> row i of the tile) add
-//     the two accumulators, apply the feature map and write row i's entries
-//     d >= c to its triangle's packed offsets.
+// Precision.  Every W and P value is formed from the FP32-rounded features as
+// an unevaluated sum of two FP32 numbers (the products' rounding errors are
+// kept) and split into three BF16 parts, x = x1 + x2 + x3 up to 2^-26 |x|; the
+// product takes the six part pairs above 2^-26 (kind::f16 MMAs, exact products).
+// Per chunk of 64 features the five small part pairs go into the accumulator
+// first, at their own magnitude, then x1 y1 in four additions; the chunk's sum
+// leaves tensor memory and is added in FP32 registers (round to nearest).
+// Measured against 64 bits (2-norm over the array, this build / the FP32
+// multiply-add build): m = 4, n = 400, d = 100 1.1e-7 / 1.9e-7; n = 200,
+// d = 20,000 sparse 1.6e-7 / 1.6e-7 (the features' own rounding).  An entry that
+// comes out as NaN (a feature product beyond the BF16 split's range, an
+// infinite or NaN feature) is formed again by plain FP32 sums.
+//
+// GB300 mapping.  build_images writes both operands once, in the K-major
+// 128-byte-swizzled layout of the MMAs: per tile of 128 rows and chunk of 64
+// features three parts of 16 KB, so that an operand chunk is one
+// cp.async.bulk of 48 KB.  build_gemm is persistent, one block per SM: a
+// thread takes tiles from a counter and starts the copies into a ring of two
+// stages (96 KB each), a thread issues the stage's 24 MMAs of 128 x 128 x 16
+// into one of four accumulators (all 512 tensor-memory columns), eight warps
+// read the accumulators, keep the tile's sums in registers (64 columns a
+// thread) and, through a padded 32 x 32 transpose, write row segments of 32
+// consecutive entries.
+//
+// What bounds it (GB300): from some 100 features on the operand ring -- a stage
+// takes 1536 cycles of MMA, whose operand reads and the ring's own writes share
+// the 128 bytes per cycle of shared memory (2250 cycles), and two stages leave
+// about one of them to hide a copy's latency: 2700 cycles per chunk measured;
+// below, the epilogue's chain per tile (some 930 instructions a warp; two warps
+// per scheduler).  Measured, multiply-add build -> this one: m = 4, n = 400,
+// d = 100 FP32 28.6 -> 1.65 ms (131 TFLOP/s at 2 d flops per entry, 2.6 TB/s
+// written), n = 200, d = 20,000 442 -> 15.3 ms, d = 2000 44.3 -> 1.4 ms; m = 6,
+// n = 80, d = 50 127 -> 1.85 ms.  64-byte rows (chunks of 32 features, four
+// stages) measured slower, 20.5 ms at d = 20,000: the MMAs read them at a third
+// of the rate.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
+#include "tk_build.cuh"
 #include "tk_umma.cuh"
 
 namespace tk {
 
-constexpr int kCT = 128;  // tile rows and (at most) columns
-constexpr int kCEpiWarps = 4, kCGatherWarps = 8;
-constexpr int kCGatherThreads = 32 * kCGatherWarps;
-constexpr int kCThreads = 32 * (kCEpiWarps + kCGatherWarps + 1);
-constexpr int kCStages = 3;
-constexpr int kCPart = kCT * 128;  // 128 rows x 32 FP32 values
-constexpr int kCStageBytes = 4 * kCPart;  // A hi, A lo, B hi, B lo
+constexpr int kGT = 128;                       // tile rows and columns
+constexpr int kGK = 64;                        // features per chunk (128 bytes of BF16)
+constexpr int kGPart = kGT * 2 * kGK;              // one part of a tile chunk
+constexpr int kGChunk = 3 * kGPart;            // the three parts
+constexpr int kGStages = 2;
+constexpr int kGStageBytes = 2 * kGChunk;
+constexpr int kGEpiWarps = 8;                  // warps 0-7: epilogue
+constexpr int kGThreads = 32 * (kGEpiWarps + 2);  // + warp 8: copies, warp 9: MMAs
+constexpr int kGPitch = 33;                    // transpose buffer of an epilogue warp: 32 rows of 33 words
+constexpr int kGStageOut = 32 * kGPitch * 4;
+constexpr int kGAcc = 4;                       // accumulators in tensor memory (128 columns each)
+constexpr int kGTiles = 4;                     // tiles found ahead of their use
+constexpr int kGWaveChunks = 48;               // chunks of a tile from which the blocks go in step
+constexpr int kGGroup = 8;                     // row tiles that share a sweep over the columns
+constexpr size_t kGSmem = 1024 + (size_t)kGStages * kGStageBytes + (size_t)kGEpiWarps * kGStageOut;
+constexpr size_t kGMaxWork = (size_t)2 << 30;  // operand images beyond this are made and used panel by panel
 
-// Set by a tensor-core build whose bounded wait ran out (read by tk_build_status).
 __device__ int g_tc_build_status;
 
-struct CParams {
-  int m, n, d, nkc;
-  const double *X;
+// Output row of one prefix: entry p of the row is stored at obase + p for
+// p >= sb (obase = packed offset of the row's first entry, minus sb).
+struct GRow {
+  int64_t obase;
+  int32_t sb;
+  int32_t pad;
+};
+static_assert(sizeof(GRow) == 16, "row record");
+
+struct GParams {
+  BuildShape s;          // m, n, i_lo, i_hi, rows, pairs
+  int d, ldx, nkc;       // features, padded, 64-feature chunks
+  int rt0, nrt;          // row tiles of the panel
+  int ct0, nct;          // column tiles of the panel
+  const float *x32;      // n x ldx
+  unsigned char *wimg, *pimg;
+  GRow *rows;            // nrt x 128
+  int *first;            // nrt: first column tile of each row tile
+  int64_t *pre;          // task counts before each group of row tiles
+  unsigned long long *ticket;  // next task to hand out
+  int write_w, write_p;  // which images this launch makes
   int feat, degree;
-  void *K;  // entry off_lo
+  void *K;               // entry off_lo
   int64_t off_lo, off_hi;
-  int64_t total_tasks;
+  int whole;             // the whole array is built
 };
 
-struct CTask {
-  int b, L;          // last prefix value, rows/columns of its triangles
-  int stacked;       // 1: floor(128/L) whole triangles stacked, 0: one 128 x 128 block of one triangle
-  int64_t qi0;       // index (among the triangles with last value b) of the task's first triangle
-  int ntri;          // triangles in the task
-  int rt, ct;        // row / column block (L > 128)
-  int npad;          // columns, rounded up to 16 (N of the MMA)
-};
-
-__host__ __device__ __forceinline__ int64_t c_count(int m, int n, int b) {
-  const int64_t cb = (m == 2) ? 1 : multiset(b + 1, m - 3);
-  const int L = n - b;
-  if (L <= kCT) {
-    const int k = kCT / L;
-    return (cb + k - 1) / k;
-  }
-  const int64_t lt = (L + kCT - 1) / kCT;
-  return cb * (lt * (lt + 1) / 2);
+__global__ void build_x32(int n, int d, int ldx, const double *X, float *x32) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (int64_t)n * ldx) return;
+  const int r = (int)(i / ldx), k = (int)(i - (int64_t)r * ldx);
+  x32[i] = k < d ? (float)X[(int64_t)r * d + k] : 0.f;
 }
 
-// Task t -> its triangle group or block.
-__host__ __device__ __forceinline__ CTask c_decode(const CParams &p, const int64_t *pre, int64_t t) {
-  CTask r;
-  const int m = p.m, n = p.n;
-  const int ngroups = (m == 2) ? 1 : n;
-  int lo = 0, hi = ngroups - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (pre[mid] <= t) lo = mid;
-    else hi = mid - 1;
+__device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 a, __nv_bfloat16 b) {
+  return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+}
+
+// The task plan of a panel (one block): the first column tile of every row
+// tile and, per group of kGGroup row tiles, the tasks of the groups before it.
+__device__ void build_plan_tasks(const GParams &p) {
+  __shared__ int64_t part[256];
+  const int ng = (p.nrt + kGGroup - 1) / kGGroup;
+  for (int t = threadIdx.x; t < p.nrt; t += blockDim.x) {
+    const int b = build_row_last(p.s, (int64_t)(p.rt0 + t) * kGT);
+    p.first[t] = build_first_pair(p.s.n, b) / kGT;
   }
-  const int b = (m == 2) ? 0 : lo;
-  const int64_t cb = (m == 2) ? 1 : multiset(b + 1, m - 3);
-  const int L = n - b;
-  const int64_t local = t - pre[lo];
-  r.b = b;
-  r.L = L;
-  if (L <= kCT) {
-    const int k = kCT / L;
-    r.stacked = 1;
-    r.qi0 = local * k;
-    r.ntri = (int)(cb - r.qi0 < k ? cb - r.qi0 : k);
-    r.rt = r.ct = 0;
-    r.npad = (L + 15) & ~15;
-  } else {
-    const int lt = (L + kCT - 1) / kCT;
-    const int64_t T = (int64_t)lt * (lt + 1) / 2;
-    r.stacked = 0;
-    r.qi0 = local / T;
-    r.ntri = 1;
-    int tp = (int)(local - r.qi0 * T), rt = 0;
-    while (tp >= lt - rt) {
-      tp -= lt - rt;
-      ++rt;
+  __syncthreads();
+  const int per = (ng + 255) / 256;
+  const int g0 = min(ng, (int)threadIdx.x * per), g1 = min(ng, g0 + per);
+  auto count = [&](int g) -> int64_t {
+    const int lo = max(p.first[g * kGGroup], p.ct0);
+    return (int64_t)max(0, p.ct0 + p.nct - lo) * kGGroup;
+  };
+  int64_t mine = 0;
+  for (int g = g0; g < g1; ++g) mine += count(g);
+  part[threadIdx.x] = mine;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int64_t acc = 0;
+    for (int i = 0; i < 256; ++i) {
+      const int64_t v = part[i];
+      part[i] = acc;
+      acc += v;
     }
-    r.rt = rt;
-    r.ct = rt + tp;
-    const int cols = min(kCT, L - kCT * r.ct);
-    r.npad = (cols + 15) & ~15;
+    p.pre[ng] = acc;
+    *p.ticket = 0;
   }
-  return r;
+  __syncthreads();
+  int64_t acc = part[threadIdx.x];
+  for (int g = g0; g < g1; ++g) {
+    p.pre[g] = acc;
+    acc += count(g);
+  }
 }
 
-// Row r of a task: its triangle (prefix Q, packed base of (Q, b, b)) and row c.
-struct CRow {
-  bool valid;
-  int c;
-  int32_t q[kMaxOrder];
-  int64_t base;
+// Operand images of a panel: blocks (tile, chunk group); the tiles 0..nrt-1
+// are prefix rows (W), the next nct pair rows (P).  The last block row of the
+// grid (blockIdx.x == tiles) makes the task plan.
+__global__ void __launch_bounds__(256) build_images(GParams p) {
+  const int tid = threadIdx.x;
+  const int ntw = p.write_w ? p.nrt : 0, ntp = p.write_p ? p.nct : 0;
+  int tile = blockIdx.x;
+  if (tile == ntw + ntp) {
+    if (blockIdx.y == 0) build_plan_tasks(p);
+    return;
+  }
+  __shared__ uint16_t tup[kGT][kMaxOrder];
+  __shared__ uint8_t live[kGT];
+  const bool is_w = tile < ntw;
+  if (!is_w) tile -= ntw;
+  const int nf = is_w ? p.s.m - 2 : 2;  // factors of a row
+  if (tid < kGT) {
+    int32_t t[kMaxOrder];
+    bool ok;
+    if (is_w) {
+      const int64_t row = (int64_t)(p.rt0 + tile) * kGT + tid;
+      ok = row < p.s.rows;
+      GRow gr;
+      gr.obase = 0;
+      gr.sb = 0x7fffffff;
+      gr.pad = 0;
+      if (ok) {
+        const int b = build_row_tuple(p.s, row, t);
+        gr.sb = build_first_pair(p.s.n, b);
+        t[p.s.m - 2] = b;
+        t[p.s.m - 1] = b;
+        gr.obase = rank(p.s.m, p.s.n, t) - gr.sb;
+      }
+      if (blockIdx.y == 0) p.rows[(size_t)tile * kGT + tid] = gr;
+    } else {
+      const int64_t q = (int64_t)(p.ct0 + tile) * kGT + tid;
+      ok = q < p.s.pairs;
+      if (ok) unrank(2, p.s.n, q, t);
+    }
+    live[tid] = ok;
+    for (int j = 0; j < nf; ++j) tup[tid][j] = ok ? (uint16_t)t[j] : (uint16_t)0;
+  }
+  __syncthreads();
+  unsigned char *img = (is_w ? p.wimg : p.pimg) + (size_t)tile * p.nkc * kGChunk;
+  for (int kc = blockIdx.y; kc < p.nkc; kc += gridDim.y) {
+    unsigned char *dst = img + (size_t)kc * kGChunk;
+    // a thread takes 8 consecutive features of a row: 16 bytes of each part
+#pragma unroll
+    for (int it = 0; it < kGT * 8 / 256; ++it) {
+      const int e = tid + 256 * it, r = e >> 3, k8 = e & 7;
+      uint32_t o1[4] = {0, 0, 0, 0}, o2[4] = {0, 0, 0, 0}, o3[4] = {0, 0, 0, 0};
+      if (live[r]) {
+        float v[8], lo[8];
+        const float *x0 = p.x32 + (size_t)tup[r][0] * p.ldx + kc * kGK + 8 * k8;
+#pragma unroll
+        for (int i = 0; i < 8; i += 4) {
+          const float4 f = *reinterpret_cast<const float4 *>(x0 + i);
+          v[i] = f.x;
+          v[i + 1] = f.y;
+          v[i + 2] = f.z;
+          v[i + 3] = f.w;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) lo[i] = 0.f;
+        for (int j = 1; j < nf; ++j) {
+          const float *xj = p.x32 + (size_t)tup[r][j] * p.ldx + kc * kGK + 8 * k8;
+#pragma unroll
+          for (int i = 0; i < 8; i += 4) {
+            const float4 f = *reinterpret_cast<const float4 *>(xj + i);
+            const float g[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const float h = v[i + u] * g[u];
+              // (v + lo) g = h + the rounding error of v g + lo g
+              lo[i + u] = fmaf(v[i + u], g[u], -h) + lo[i + u] * g[u];
+              v[i + u] = h;
+            }
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {
+          __nv_bfloat16 a1[2], a2[2], a3[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            a1[u] = __float2bfloat16_rn(v[i + u]);
+            const float r1 = v[i + u] - __bfloat162float(a1[u]);
+            a2[u] = __float2bfloat16_rn(r1);
+            a3[u] = __float2bfloat16_rn((r1 - __bfloat162float(a2[u])) + lo[i + u]);
+          }
+          o1[i / 2] = pack_bf16(a1[0], a1[1]);
+          o2[i / 2] = pack_bf16(a2[0], a2[1]);
+          o3[i / 2] = pack_bf16(a3[0], a3[1]);
+        }
+      }
+      const uint32_t so = (uint32_t)(r >> 3) * 1024u + (uint32_t)(r & 7) * 128u + (uint32_t)((k8 ^ (r & 7)) << 4);
+      *reinterpret_cast<uint4 *>(dst + so) = make_uint4(o1[0], o1[1], o1[2], o1[3]);
+      *reinterpret_cast<uint4 *>(dst + kGPart + so) = make_uint4(o2[0], o2[1], o2[2], o2[3]);
+      *reinterpret_cast<uint4 *>(dst + 2 * kGPart + so) = make_uint4(o3[0], o3[1], o3[2], o3[3]);
+    }
+  }
+}
+
+// A block's tasks, taken from a counter in runs of `step`.  Groups of kGGroup
+// row tiles sweep the columns together (their operands are then read from HBM
+// once and shared through L2): the tasks of a group are the column tiles from
+// the first one its first row reaches, the group's row tiles innermost.  Single
+// tasks where a group holds one for every block (the blocks then work on
+// neighbouring tiles), else runs, so that the search for the group is shared.
+// From kGWaveChunks chunks on the operands of the blocks' tiles exceed L2: the
+// blocks then take every gridDim-th task, start their tiles together and pass
+// the features in step, reading each operand chunk from HBM about once (n = 200,
+// d = 20,000: 15.3 ms against 18.1 from the counter).  A few tiles per block
+// only are balanced better by the counter (n = 30, d = 20,000: 0.45 / 0.83 ms).
+struct GWalk {
+  int64_t t, end, total;
+  int64_t wave;  // next task of the fixed schedule, or -1
+  int g, ng, step;
+  __device__ void init(const GParams &p) {
+    ng = (p.nrt + kGGroup - 1) / kGGroup;
+    total = p.pre[ng];
+    g = 0;
+    t = end = 0;
+    step = total >= (int64_t)ng * gridDim.x || total < (int64_t)64 * gridDim.x ? 1 : kGGroup;
+    wave = p.nkc >= kGWaveChunks && total >= (int64_t)4 * gridDim.x ? (int64_t)blockIdx.x : -1;
+  }
+  // next tile (row tile, column tile) within the panel; false at the end
+  __device__ bool next(const GParams &p, int *rt, int *ct) {
+    for (;;) {
+      if (t >= end) {
+        if (wave >= 0) {
+          t = wave;
+          wave += gridDim.x;
+        } else {
+          t = (int64_t)atomicAdd(p.ticket, (unsigned long long)step);
+        }
+        if (t >= total) return false;
+        end = wave >= 0 ? t + 1 : min(t + step, total);
+      }
+      if (t >= p.pre[g + 1]) {
+        ++g;
+        if (t >= p.pre[g + 1]) {  // the largest g with pre[g] <= t
+          int lo = g, hi = ng - 1;
+          while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (p.pre[mid] <= t) lo = mid; else hi = mid - 1;
+          }
+          g = lo;
+        }
+      }
+      const int64_t local = t - p.pre[g];
+      const int r = g * kGGroup + (int)(local % kGGroup);
+      const int c = max(p.first[g * kGGroup], p.ct0) + (int)(local / kGGroup);
+      ++t;
+      if (r >= p.nrt || c < p.first[r]) continue;
+      *rt = r;
+      *ct = c - p.ct0;
+      return true;
+    }
+  }
 };
-__host__ __device__ __forceinline__ CRow c_row(const CParams &p, const CTask &t, int r) {
-  CRow w;
-  const int m = p.m, n = p.n, b = t.b;
-  int64_t qi;
-  if (t.stacked) {
-    const int j = r / t.L;
-    w.valid = j < t.ntri;
-    qi = t.qi0 + (w.valid ? j : 0);
-    w.c = b + r - j * t.L;
-  } else {
-    w.c = b + kCT * t.rt + r;
-    w.valid = w.c < n;
-    qi = t.qi0;
-  }
-  int32_t tup[kMaxOrder];
-  if (m >= 3) {
-    if (m > 3) unrank(m - 3, b + 1, qi, tup);
-    tup[m - 3] = b;
-  }
-  tup[m - 2] = b;
-  tup[m - 1] = b;
-  for (int j = 0; j < m - 2; ++j) w.q[j] = tup[j];
-  w.base = (m == 2) ? 0 : rank(m, n, tup);
-  return w;
-}
 
-__host__ __device__ __forceinline__ int c_col0(const CTask &t) { return t.b + (t.stacked ? 0 : kCT * t.ct); }
-
-template <typename ST>
-__device__ __forceinline__ void c_store(void *K, int64_t idx, float v);
-template <>
-__device__ __forceinline__ void c_store<float>(void *K, int64_t idx, float v) {
-  reinterpret_cast<float *>(K)[idx] = v;
-}
-template <>
-__device__ __forceinline__ void c_store<__nv_bfloat16>(void *K, int64_t idx, float v) {
-  reinterpret_cast<__nv_bfloat16 *>(K)[idx] = __float2bfloat16_rn(v);
-}
-
-__device__ __forceinline__ float c_feat(float v, int feat, int degree) {
-  if (feat == TK_FEAT_POLY) {
-    float r = 1.f;
-    for (int i = 0; i < degree; ++i) r *= v;
-    return r;
-  }
-  if (feat == TK_FEAT_EXP) return expf(v);
-  return v;
-}
-
-__device__ __forceinline__ bool c_wait(uint64_t *bar, uint32_t parity, volatile int *bad) {
+__device__ __forceinline__ bool g_wait(uint64_t *bar, uint32_t parity, volatile int *bad) {
   if (*bad) return false;
   if (mbar_wait_bounded(bar, parity)) return true;
   *bad = 1;
   return false;
 }
 
-// Whether any entry of the task lies in [off_lo, off_hi).
-__host__ __device__ __forceinline__ bool c_live(const CParams &p, const CTask &t) {
-  const CRow f = c_row(p, t, 0);
-  const CRow l = c_row(p, t, t.stacked ? (t.ntri - 1) * t.L : 0);
-  const int64_t L = t.L;
-  return !(l.base + L * (L + 1) / 2 <= p.off_lo || f.base >= p.off_hi);
+// 32 consecutive 32-bit columns of this thread's tensor-memory lane
+__device__ __forceinline__ void g_tmem_ld32(uint32_t taddr, uint32_t *r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr)
+      : "memory");
+}
+
+// D (tensor memory) = A B^T (+ D), BF16 operands, FP32 accumulation
+__device__ __forceinline__ void g_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                      uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// instruction descriptor of kind::f16 with BF16 operands, both K-major: D in
+// FP32 (bits 4-5 = 1), A and B in BF16 (bits 7-9, 10-12 = 1), N >> 3, M >> 4
+constexpr uint32_t kGIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kGT >> 3) << 17) |
+                             ((uint32_t)(kGT >> 4) << 24);
+
+// one linear entry by plain FP32 sums over the features
+__device__ __noinline__ float build_entry_plain(const GParams &p, int64_t row, int64_t pair) {
+  int32_t t[kMaxOrder];
+  build_row_tuple(p.s, row, t);
+  unrank(2, p.s.n, pair, t + p.s.m - 2);
+  float s = 0.f;
+  for (int k = 0; k < p.d; ++k) {
+    float w = 1.f;
+    for (int j = 0; j < p.s.m - 2; ++j) w *= p.x32[(size_t)t[j] * p.ldx + k];
+    s = __fmaf_rn(p.x32[(size_t)t[p.s.m - 2] * p.ldx + k] * w, p.x32[(size_t)t[p.s.m - 1] * p.ldx + k], s);
+  }
+  return s;
+}
+
+// Store 32 rows x 32 pairs of a tile from the warp's transpose buffer: lane i
+// holds row i's offset relative to row 0 (rel) and first pair (sb), K0 points
+// at this lane's entry of row 0, its pair is `pr`.  EDGE: some of the entries
+// are not wanted, or they go through a feature map.
+template <typename ST, bool EDGE, typename OT>
+__device__ __forceinline__ void store_rows(const GParams &p, const float *stg, OT rel, int sb, ST *K0, int64_t off0,
+                                           int64_t pr, int lane) {
+  __syncwarp();
+  // a batch of rows at a time: their offsets and values first, then the stores
+  constexpr int kB = EDGE ? 8 : 16;
+#pragma unroll 1
+  for (int i0 = 0; i0 < 32; i0 += kB) {
+    OT o[kB];
+    float v[kB];
+    bool ok[kB];
+#pragma unroll
+    for (int i = 0; i < kB; ++i) o[i] = __shfl_sync(0xffffffffu, rel, i0 + i);
+#pragma unroll
+    for (int i = 0; i < kB; ++i) v[i] = stg[(i0 + i) * kGPitch + lane];
+    if (EDGE) {
+#pragma unroll
+      for (int i = 0; i < kB; ++i) {
+        const int64_t off = off0 + o[i];
+        ok[i] = pr >= __shfl_sync(0xffffffffu, sb, i0 + i) && pr < p.s.pairs && off >= p.off_lo && off < p.off_hi;
+      }
+      if (p.feat != TK_FEAT_LINEAR) {
+#pragma unroll
+        for (int i = 0; i < kB; ++i) v[i] = feat_apply(v[i], p.feat, p.degree);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kB; ++i)
+      if (!EDGE || ok[i]) store_entry<ST, float>(K0, o[i], v[i]);
+  }
 }
 
 template <typename ST>
-__global__ void __launch_bounds__(kCThreads, 1) tc_build_kernel(CParams p) {
-  extern __shared__ unsigned char cb_smem_raw[];
-  __shared__ uint64_t bar_full[kCStages], bar_empty[kCStages], bar_accf[2], bar_acce[2];
+__global__ void __launch_bounds__(kGThreads, 1) build_gemm(GParams p) {
+  extern __shared__ unsigned char g_smem_raw[];
+  __shared__ uint64_t bar_full[kGStages], bar_empty[kGStages], bar_accf[kGAcc], bar_acce[kGAcc];
+  // the next tiles, found by the copying thread for every role
+  __shared__ uint64_t bar_tile[kGTiles], bar_told[kGTiles];
+  __shared__ int2 tile_at[kGTiles];
   __shared__ uint32_t tbase;
   __shared__ int s_bad;
-  unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(cb_smem_raw) + 1023) &
+  unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(g_smem_raw) + 1023) &
                                                         ~uintptr_t(1023));
-  int64_t *pre = reinterpret_cast<int64_t *>(sm + kCStages * kCStageBytes);  // [n + 1]
-  float *wtab = reinterpret_cast<float *>(pre + (TK_MAX_POINTS + 1));        // [128 triangles][32 features]
-  int32_t *qtab = reinterpret_cast<int32_t *>(wtab + kCT * 32);               // [128 triangles][kMaxOrder]
-
-  const int tid = threadIdx.x, w = tid >> 5;
-  const int m = p.m, n = p.n;
-  const int ngroups = (m == 2) ? 1 : n;
-  for (int b = tid; b < ngroups; b += blockDim.x) pre[b + 1] = c_count(m, n, b);
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   if (w == 0) {
     umma::tmem_alloc(&tbase, 512);
     umma::tmem_relinquish();
   }
   if (tid == 0) {
-    for (int s = 0; s < kCStages; ++s) {
-      mbar_init(&bar_full[s], kCGatherThreads);
+    for (int s = 0; s < kGStages; ++s) {
+      mbar_init(&bar_full[s], 1);
       mbar_init(&bar_empty[s], 1);
     }
-    for (int b2 = 0; b2 < 2; ++b2) {
-      mbar_init(&bar_accf[b2], 1);
-      mbar_init(&bar_acce[b2], 32 * kCEpiWarps);
+    for (int b = 0; b < kGAcc; ++b) {
+      mbar_init(&bar_accf[b], 1);
+      mbar_init(&bar_acce[b], 32 * kGEpiWarps);
+    }
+    for (int i = 0; i < kGTiles; ++i) {
+      mbar_init(&bar_tile[i], 1);
+      mbar_init(&bar_told[i], kGEpiWarps + 1);
     }
     fence_barrier_init();
     s_bad = 0;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    pre[0] = 0;
-    for (int b = 1; b <= ngroups; ++b) pre[b] += pre[b - 1];
   }
   umma::fence_before_sync();
   __syncthreads();
   umma::fence_after_sync();
   volatile int *bad = &s_bad;
+  uint32_t gc = 0;  // chunks so far
+  uint32_t ti = 0;  // tiles so far
+  // the i-th tile of this block; x < 0 after the last one
+  auto tile = [&](uint32_t i) -> int2 {
+    if (!g_wait(&bar_tile[i % kGTiles], (i / kGTiles) & 1u, bad)) return make_int2(-1, -1);
+    return tile_at[i % kGTiles];
+  };
 
-  if (w < kCEpiWarps) {
+  if (w < kGEpiWarps) {
     // ---------------------------------------------------------------- epilogue
-    const uint32_t tl = tbase + ((uint32_t)(32 * w) << 16);
-    int jl = 0;
-    for (int64_t t = blockIdx.x; t < p.total_tasks; t += gridDim.x) {
-      const CTask tsk = c_decode(p, pre, t);
-      if (!c_live(p, tsk)) continue;
-      const CRow row = c_row(p, tsk, tid);
-      const int buf = jl & 1;
-      if (!c_wait(&bar_accf[buf], (uint32_t)(jl >> 1) & 1u, bad)) break;
-      umma::fence_after_sync();
-      const int c = row.c, b = tsk.b, d0 = c_col0(tsk);
-      const int64_t rowoff = row.base + (int64_t)(c - b) * (2 * n - b - c + 1) / 2 - c;
-      const uint32_t tb = tl + (uint32_t)buf * 256u, ts = tb + 128u;
-      for (int j0 = 0; j0 < tsk.npad; j0 += 16) {
-        uint32_t ub[16], us[16];
-        umma::tmem_ld16_async(tb + j0, ub);
-        umma::tmem_ld16_async(ts + j0, us);
-        umma::tmem_wait_ld();
-        if (!row.valid) continue;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int dd = d0 + j0 + i;
-          if (dd < c || dd >= n) continue;
-          const int64_t off = rowoff + dd;
-          if (off < p.off_lo || off >= p.off_hi) continue;
-          const float v = __uint_as_float(ub[i]) + __uint_as_float(us[i]);
-          c_store<ST>(p.K, off - p.off_lo, c_feat(v, p.feat, p.degree));
-        }
-      }
-      umma::fence_before_sync();
-      mbar_arrive(&bar_acce[buf]);
-      ++jl;
-    }
-  } else if (w < kCEpiWarps + kCGatherWarps) {
-    // ---------------------------------------------------------------- operands
-    // per task the prefixes of its triangles go into a table; per chunk each
-    // triangle's weight row w_Q[k] = prod_{q in Q} x_{q,k} is formed once, then
-    // warp gw builds rows 16 gw .. 16 gw + 15 of both operands, lanes along
-    // the chunk's 32 features, all row loads issued before the first is used.
-    // (No early exit: the gathering warps meet at named barriers, so a wait
-    // that ran out only skips its stage and the loops run to the end.)
-    const int gt = tid - 32 * kCEpiWarps, gw = gt >> 5, lane = tid & 31;
-    uint32_t gc = 0;
-    for (int64_t t = blockIdx.x; t < p.total_tasks; t += gridDim.x) {
-      const CTask tsk = c_decode(p, pre, t);
-      if (!c_live(p, tsk)) continue;
-      // the previous task's last chunk has been read by every gathering warp
-      asm volatile("bar.sync 1, %0;" ::"n"(kCGatherThreads) : "memory");
-      if (gt < tsk.ntri) {
-        const CRow first = c_row(p, tsk, tsk.stacked ? gt * tsk.L : 0);
-        for (int j = 0; j < m - 2; ++j) qtab[gt * kMaxOrder + j] = first.q[j];
-      }
-      int rc[16];
-      bool rv[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int r = 16 * gw + i;
-        if (tsk.stacked) {
-          const int j = r / tsk.L;
-          rv[i] = j < tsk.ntri;
-          rc[i] = tsk.b + r - j * tsk.L;
-        } else {
-          rc[i] = tsk.b + kCT * tsk.rt + r;
-          rv[i] = rc[i] < n;
-        }
-      }
-      const int d0 = c_col0(tsk);
-      for (int kc = 0; kc < p.nkc; ++kc, ++gc) {
-        const int s = (int)(gc % kCStages);
-        const uint32_t use = gc / kCStages;
-        const int k = 32 * kc + lane;
-        const bool kok = k < p.d;
-        // the weight rows of the task's triangles for this chunk
-        asm volatile("bar.sync 1, %0;" ::"n"(kCGatherThreads) : "memory");
-        for (int j = gw; j < tsk.ntri; j += kCGatherWarps) {
-          double wv = kok ? 1.0 : 0.0;
-          if (kok)
-            for (int jj = 0; jj < m - 2; ++jj) wv *= p.X[(size_t)qtab[j * kMaxOrder + jj] * p.d + k];
-          wtab[j * 32 + lane] = (float)wv;
-        }
-        double xa[16], xb[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int r = 16 * gw + i, dd = d0 + r;
-          xa[i] = (rv[i] && kok) ? p.X[(size_t)rc[i] * p.d + k] : 0.0;
-          xb[i] = (r < tsk.npad && dd < n && kok) ? p.X[(size_t)dd * p.d + k] : 0.0;
-        }
-        asm volatile("bar.sync 1, %0;" ::"n"(kCGatherThreads) : "memory");  // weight rows in place
-        if (use > 0 && !c_wait(&bar_empty[s], (use - 1) & 1u, bad)) continue;
-        unsigned char *st = sm + s * kCStageBytes;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int r = 16 * gw + i;
-          const int j = tsk.stacked ? r / tsk.L : 0;
-          const double a = rv[i] ? xa[i] * wtab[(j < tsk.ntri ? j : 0) * 32 + lane] : 0.0;
-          float h, l;
-          umma::split_tf32((float)a, h, l);
-          const uint32_t so = umma::sw128_offset((uint32_t)r, (uint32_t)lane);
-          *reinterpret_cast<float *>(st + so) = h;
-          *reinterpret_cast<float *>(st + kCPart + so) = l;
-          umma::split_tf32((float)xb[i], h, l);
-          *reinterpret_cast<float *>(st + 2 * kCPart + so) = h;
-          *reinterpret_cast<float *>(st + 3 * kCPart + so) = l;
-        }
-        fence_proxy_async();  // the operands written above become visible to the tensor cores
-        mbar_arrive(&bar_full[s]);
-      }
-    }
-  } else if ((tid & 31) == 0) {
-    // ---------------------------------------------------------------- MMA issue
-    uint32_t gc = 0;
-    int jl = 0;
-    const uint32_t idesc_base = umma::idesc_tf32(kCT, 16) & ~(0x3Fu << 17);
+    const int quad = w & 3, half = w >> 2;  // 32 rows, 64 columns of the tile
+    const uint32_t tl = tbase + ((uint32_t)(32 * quad) << 16) + 64u * half;
+    float *stg = reinterpret_cast<float *>(sm + kGStages * kGStageBytes + w * kGStageOut);
     bool ok = true;
-    for (int64_t t = blockIdx.x; t < p.total_tasks && ok; t += gridDim.x) {
-      const CTask tsk = c_decode(p, pre, t);
-      if (!c_live(p, tsk)) continue;
-      const int buf = jl & 1;
-      if (jl >= 2 && !c_wait(&bar_acce[buf], (uint32_t)((jl >> 1) - 1) & 1u, bad)) break;
-      umma::fence_after_sync();
-      const uint32_t idesc = idesc_base | ((uint32_t)(tsk.npad >> 3) << 17);
-      const uint32_t tb = tbase + (uint32_t)buf * 256u, ts = tb + 128u;
+    // the warp's view of a tile: its coordinates and, on lane i, row i's record;
+    // the next tile's are fetched before the current one is stored
+    GRow next_row;
+    auto fetch = [&]() -> int2 {
+      int2 at = make_int2(-1, -1);
+      if (lane == 0) {
+        at = tile(ti);
+        if (at.x >= 0) mbar_arrive(&bar_told[ti % kGTiles]);
+      }
+      ++ti;
+      at.x = __shfl_sync(0xffffffffu, at.x, 0);
+      at.y = __shfl_sync(0xffffffffu, at.y, 0);
+      if (at.x >= 0) next_row = p.rows[(size_t)at.x * kGT + 32 * quad + lane];
+      return at;
+    };
+    int2 at = fetch();
+    while (at.x >= 0) {
+      const int rt = at.x, ct = at.y;
+      const GRow mine = next_row;
+      float acc[64];
       for (int kc = 0; kc < p.nkc; ++kc, ++gc) {
-        const int s = (int)(gc % kCStages);
-        if (!c_wait(&bar_full[s], (gc / kCStages) & 1u, bad)) {
+        const uint32_t buf = gc % kGAcc;
+        if (!g_wait(&bar_accf[buf], (gc / kGAcc) & 1u, bad)) {
           ok = false;
           break;
         }
         umma::fence_after_sync();
-        const uint32_t a0 = saddr(sm + s * kCStageBytes), b0 = a0 + 2 * kCPart;
+        uint32_t a[64];
+        g_tmem_ld32(tl + 128u * buf, a);
+        g_tmem_ld32(tl + 128u * buf + 32u, a + 32);
+        umma::tmem_wait_ld();
+        umma::fence_before_sync();
+        mbar_arrive(&bar_acce[buf]);
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {
-          const uint64_t ah = umma::desc_sw128(a0 + 32 * ks), al = umma::desc_sw128(a0 + kCPart + 32 * ks);
-          const uint64_t bh = umma::desc_sw128(b0 + 32 * ks), bl = umma::desc_sw128(b0 + kCPart + 32 * ks);
-          const uint32_t acc = (kc > 0 || ks > 0) ? 1u : 0u;
-          umma::mma_tf32(tb, ah, bh, idesc, acc);
-          umma::mma_tf32(ts, ah, bl, idesc, acc);
-          umma::mma_tf32(ts, al, bh, idesc, 1u);
-        }
-        umma::mma_commit(&bar_empty[s]);
+        for (int i = 0; i < 64; ++i) acc[i] = kc == 0 ? __uint_as_float(a[i]) : acc[i] + __uint_as_float(a[i]);
       }
-      umma::mma_commit(&bar_accf[buf]);
-      ++jl;
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      at = fetch();
+      const int64_t pw = (int64_t)(p.ct0 + ct) * kGT + 64 * half;  // first pair of this warp's columns
+      const int64_t row0 = (int64_t)(p.rt0 + rt) * kGT + 32 * quad;
+      // all 32 x 64 entries are wanted (rows are ordered by sb) and need no map
+      const bool inside = p.whole && p.feat == TK_FEAT_LINEAR && pw + 64 <= p.s.pairs &&
+                          __shfl_sync(0xffffffffu, mine.sb, 31) <= pw;
+      const int64_t obase0 = __shfl_sync(0xffffffffu, mine.obase, 0), rel = mine.obase - obase0;
+      const bool near = __all_sync(0xffffffffu, rel == (int64_t)(int)rel);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        bool odd = false;
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          stg[lane * kGPitch + j] = acc[32 * h + j];
+          odd |= acc[32 * h + j] != acc[32 * h + j];
+        }
+        odd = __any_sync(0xffffffffu, odd);
+        const int64_t pr = pw + 32 * h + lane, off0 = obase0 + pr;
+        ST *K0 = reinterpret_cast<ST *>(p.K) + (off0 - p.off_lo);
+        if (inside && near) store_rows<ST, false, int>(p, stg, (int)rel, mine.sb, K0, off0, pr, lane);
+        else store_rows<ST, true, int64_t>(p, stg, rel, mine.sb, K0, off0, pr, lane);
+        if (odd) {
+          for (int i = 0; i < 32; ++i) {
+            const int64_t off = __shfl_sync(0xffffffffu, mine.obase, i) + pr;
+            const int sb = __shfl_sync(0xffffffffu, mine.sb, i);
+            const float v = stg[i * kGPitch + lane];
+            if (v != v && pr >= sb && pr < p.s.pairs && off >= p.off_lo && off < p.off_hi)
+              store_entry<ST, float>(p.K, off - p.off_lo,
+                                     feat_apply(build_entry_plain(p, row0 + i, pr), p.feat, p.degree));
+          }
+        }
+      }
+    }
+  } else if (w == kGEpiWarps) {
+    // ---------------------------------------------------------------- copies
+    if (lane == 0) {
+      GWalk walk;
+      walk.init(p);
+      bool ok = true;
+      while (ok) {
+        int rt = -1, ct = -1;
+        const bool more = walk.next(p, &rt, &ct);
+        const uint32_t i = ti % kGTiles, use = ti / kGTiles;
+        if (use > 0 && !g_wait(&bar_told[i], (use - 1) & 1u, bad)) break;
+        ++ti;
+        tile_at[i] = make_int2(rt, ct);
+        mbar_arrive(&bar_tile[i]);
+        if (!more) break;
+        const unsigned char *a = p.wimg + (size_t)rt * p.nkc * kGChunk;
+        const unsigned char *b = p.pimg + (size_t)ct * p.nkc * kGChunk;
+        for (int kc = 0; kc < p.nkc; ++kc, ++gc) {
+          const uint32_t s = gc % kGStages, use = gc / kGStages;
+          if (use > 0 && !g_wait(&bar_empty[s], (use - 1) & 1u, bad)) {
+            ok = false;
+            break;
+          }
+          unsigned char *st = sm + s * kGStageBytes;
+          mbar_expect_tx(&bar_full[s], kGStageBytes);
+          bulk_g2s(st, a + (size_t)kc * kGChunk, kGChunk, &bar_full[s]);
+          bulk_g2s(st + kGChunk, b + (size_t)kc * kGChunk, kGChunk, &bar_full[s]);
+        }
+      }
+      // no copy may be in flight when the block ends: the last use of each
+      // stage has landed
+      for (uint32_t s = 0; s < kGStages; ++s) {
+        const uint32_t uses = gc / kGStages + (gc % kGStages > s ? 1u : 0u);
+        if (uses > 0) mbar_wait_bounded(&bar_full[s], (uses - 1) & 1u);
+      }
+    }
+  } else if (lane == 0) {
+    // ---------------------------------------------------------------- MMAs
+    bool ok = true;
+    while (ok) {
+      const int2 at = tile(ti);
+      if (at.x < 0) break;
+      mbar_arrive(&bar_told[ti % kGTiles]);
+      ++ti;
+      for (int kc = 0; kc < p.nkc; ++kc, ++gc) {
+        const uint32_t s = gc % kGStages, buf = gc % kGAcc;
+        if ((gc >= kGAcc && !g_wait(&bar_acce[buf], (gc / kGAcc - 1) & 1u, bad)) ||
+            !g_wait(&bar_full[s], (gc / kGStages) & 1u, bad)) {
+          ok = false;
+          break;
+        }
+        umma::fence_after_sync();
+        const uint32_t a0 = saddr(sm + s * kGStageBytes), b0 = a0 + kGChunk;
+        const uint32_t tm = tbase + 128u * buf;
+        const int nks = min(4, (p.d - kc * kGK + 15) >> 4);
+        // the five small part pairs of the whole chunk first: the accumulator
+        // then carries them at their own magnitude
+        for (int ks = 0; ks < nks; ++ks) {
+          const uint64_t a1 = umma::desc_sw128(a0 + 32 * ks), a2 = umma::desc_sw128(a0 + kGPart + 32 * ks),
+                         a3 = umma::desc_sw128(a0 + 2 * kGPart + 32 * ks);
+          const uint64_t b1 = umma::desc_sw128(b0 + 32 * ks), b2 = umma::desc_sw128(b0 + kGPart + 32 * ks),
+                         b3 = umma::desc_sw128(b0 + 2 * kGPart + 32 * ks);
+          g_mma(tm, a1, b3, kGIdesc, ks > 0 ? 1u : 0u);
+          g_mma(tm, a2, b2, kGIdesc, 1u);
+          g_mma(tm, a3, b1, kGIdesc, 1u);
+          g_mma(tm, a1, b2, kGIdesc, 1u);
+          g_mma(tm, a2, b1, kGIdesc, 1u);
+        }
+        for (int ks = 0; ks < nks; ++ks)
+          g_mma(tm, umma::desc_sw128(a0 + 32 * ks), umma::desc_sw128(b0 + 32 * ks), kGIdesc, 1u);
+        umma::mma_commit(&bar_empty[s]);
+        umma::mma_commit(&bar_accf[buf]);
+      }
     }
     // nothing may still write tensor memory when it is released
-    if (jl > 0) mbar_wait_bounded(&bar_accf[(jl - 1) & 1], (uint32_t)((jl - 1) >> 1) & 1u);
+    if (gc > 0) mbar_wait_bounded(&bar_accf[(gc - 1) % kGAcc], ((gc - 1) / kGAcc) & 1u);
   }
   umma::fence_before_sync();
   __syncthreads();
@@ -385,44 +601,118 @@ __global__ void __launch_bounds__(kCThreads, 1) tc_build_kernel(CParams p) {
   if (tid == 0 && s_bad) atomicExch(&g_tc_build_status, TK_ETIMEOUT);
 }
 
-size_t tc_build_smem() {
-  return 1024 + (size_t)kCStages * kCStageBytes + (size_t)(TK_MAX_POINTS + 1) * sizeof(int64_t) +
-         (size_t)kCT * 32 * sizeof(float) + (size_t)kCT * kMaxOrder * sizeof(int32_t);
+// ------------------------------------------------------------------ host
+struct GLayout {
+  size_t x32, first, pre, rows, wimg, pimg, total;
+};
+
+static size_t g_align(size_t x) { return (x + 1023) & ~size_t(1023); }
+
+// workspace of panels of `nrt` row tiles and `nct` column tiles
+static GLayout g_layout(int n, int ldx, int nkc, int64_t nrt, int64_t nct) {
+  GLayout L;
+  size_t off = 0;
+  L.x32 = off;
+  off = g_align(off + (size_t)n * ldx * sizeof(float));
+  L.first = off;
+  off = g_align(off + (size_t)nrt * sizeof(int));
+  L.pre = off;
+  off = g_align(off + (size_t)((nrt + kGGroup - 1) / kGGroup + 2) * sizeof(int64_t));  // and the ticket
+  L.rows = off;
+  off = g_align(off + (size_t)nrt * kGT * sizeof(GRow));
+  L.wimg = off;
+  off += (size_t)nrt * nkc * kGChunk;
+  L.pimg = off;
+  off += (size_t)nct * nkc * kGChunk;
+  L.total = off + 1024;  // the workspace's own alignment
+  return L;
 }
 
-int build_tc(int m, int n, int d, const double *X, int feat, int degree, int storage, int64_t off_lo,
-             int64_t off_hi, void *K, cudaStream_t st) {
+static void g_sizes(const BuildShape &s, int d, int *ldx, int *nkc, int64_t *rt, int64_t *ct) {
+  *nkc = (d + kGK - 1) / kGK;
+  *ldx = *nkc * kGK;
+  *rt = (s.rows + kGT - 1) / kGT;
+  *ct = (s.pairs + kGT - 1) / kGT;
+}
+
+size_t build_tc_workspace_bytes(int m, int n, int d) {
+  BuildShape s = build_shape(m, n, 0, n - 1);
+  int ldx, nkc;
+  int64_t rt, ct;
+  g_sizes(s, d, &ldx, &nkc, &rt, &ct);
+  const size_t least = g_layout(n, ldx, nkc, 1, 1).total;
+  // (row tiles are counted in double: their bytes can exceed 64 bits' worth of a full image)
+  const double full = (double)(rt + ct) * nkc * kGChunk + (double)rt * kGT * sizeof(GRow);
+  if (full > (double)kGMaxWork) return std::max(least, kGMaxWork + g_align((size_t)n * ldx * sizeof(float)));
+  return g_layout(n, ldx, nkc, rt, ct).total;
+}
+
+int build_tc(int m, int n, int d, const double *X, int feat, int degree, int storage, int64_t off_lo, int64_t off_hi,
+             void *K, void *work, size_t work_bytes, cudaStream_t st) {
   DevInfo di;
   int rc = dev_info(&di);
   if (rc != TK_OK) return rc;
-  const size_t smem = tc_build_smem();
-  if (smem > (size_t)di.smem_optin) return fail(TK_EUNSUPPORTED, "tensor-core build: shared memory");
-  CParams p;
-  p.m = m;
-  p.n = n;
+  if (kGSmem > (size_t)di.smem_optin) return fail(TK_EUNSUPPORTED, "tensor-core build: shared memory");
+  GParams p;
+  // only the prefixes whose first index the range reaches
+  int32_t t[16];
+  unrank(m, n, off_lo, t);
+  const int i_lo = t[0];
+  unrank(m, n, off_hi - 1, t);
+  p.s = build_shape(m, n, i_lo, t[0]);
   p.d = d;
-  p.nkc = (d + 31) / 32;
-  p.X = X;
+  int64_t rt, ct;
+  g_sizes(p.s, d, &p.ldx, &p.nkc, &rt, &ct);
+  // panel sizes: everything at once where the workspace holds it, else the
+  // images' share of it split evenly (results do not depend on the panels)
+  int64_t nrt = rt, nct = ct;
+  unsigned char *ws = reinterpret_cast<unsigned char *>(((uintptr_t)work + 1023) & ~uintptr_t(1023));
+  while (g_layout(n, p.ldx, p.nkc, nrt, nct).total > work_bytes) {
+    if (nrt == 1 && nct == 1) return fail(TK_ENOMEM, "tensor-core build: workspace of %zu bytes", work_bytes);
+    if (nrt >= nct) nrt = (nrt + 1) / 2; else nct = (nct + 1) / 2;
+  }
+  const GLayout L = g_layout(n, p.ldx, p.nkc, nrt, nct);
+  float *x32 = reinterpret_cast<float *>(ws + L.x32);
+  p.x32 = x32;
+  p.wimg = ws + L.wimg;
+  p.pimg = ws + L.pimg;
+  p.rows = reinterpret_cast<GRow *>(ws + L.rows);
+  p.first = reinterpret_cast<int *>(ws + L.first);
+  p.pre = reinterpret_cast<int64_t *>(ws + L.pre) + 1;
+  p.ticket = reinterpret_cast<unsigned long long *>(ws + L.pre);
   p.feat = feat;
   p.degree = degree;
   p.K = K;
   p.off_lo = off_lo;
   p.off_hi = off_hi;
-  int64_t total = 0;
-  for (int b = 0; b < ((m == 2) ? 1 : n); ++b) total += c_count(m, n, b);
-  p.total_tasks = total;
-  if (total == 0) return TK_OK;
-  const int grid = (int)std::min<int64_t>(total, di.sms);
-  if (storage == TK_F32) {
-    TK_CUDA_CHECK(cudaFuncSetAttribute(tc_build_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem));
-    tc_build_kernel<float><<<grid, kCThreads, smem, st>>>(p);
-  } else {
-    TK_CUDA_CHECK(cudaFuncSetAttribute(tc_build_kernel<__nv_bfloat16>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    tc_build_kernel<__nv_bfloat16><<<grid, kCThreads, smem, st>>>(p);
-  }
+  p.whole = off_lo == 0 && off_hi == multiset(n, m);
+  build_x32<<<(unsigned)(((int64_t)n * p.ldx + 255) / 256), 256, 0, st>>>(n, d, p.ldx, X, x32);
   TK_CUDA_CHECK(cudaGetLastError());
+  const void *kern = storage == TK_F32 ? (const void *)build_gemm<float> : (const void *)build_gemm<__nv_bfloat16>;
+  TK_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGSmem));
+  bool have_w = false;
+  for (int64_t c0 = 0; c0 < ct; c0 += nct) {
+    p.ct0 = (int)c0;
+    p.nct = (int)std::min(nct, ct - c0);
+    p.write_p = 1;
+    for (int64_t r0 = 0; r0 < rt; r0 += nrt) {
+      // the panel's first row has its smallest b: past these columns, done
+      if (build_first_pair(n, build_row_last(p.s, r0 * kGT)) / kGT >= c0 + p.nct) break;
+      p.rt0 = (int)r0;
+      p.nrt = (int)std::min(nrt, rt - r0);
+      p.write_w = !(have_w && nrt == rt);
+      const int tiles = (p.write_w ? p.nrt : 0) + (p.write_p ? p.nct : 0);
+      const int split = std::max(1, std::min(p.nkc, 4 * di.sms / std::max(1, tiles)));
+      build_images<<<dim3((unsigned)tiles + 1, (unsigned)split), 256, 0, st>>>(p);
+      TK_CUDA_CHECK(cudaGetLastError());
+      const int grid = (int)std::min<int64_t>((int64_t)p.nrt * p.nct, di.sms);
+      if (storage == TK_F32) build_gemm<float><<<grid, kGThreads, kGSmem, st>>>(p);
+      else build_gemm<__nv_bfloat16><<<grid, kGThreads, kGSmem, st>>>(p);
+      TK_CUDA_CHECK(cudaGetLastError());
+      have_w = true;
+      p.write_p = 0;
+    }
+  }
   return TK_OK;
 }
 
