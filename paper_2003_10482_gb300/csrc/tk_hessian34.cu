@@ -1,0 +1,344 @@
+// Full Hessian of the tensor-kernel term at orders m = 3 and 4: Hk = K[a^{m-2}]
+// as a dense n x n matrix from one pass over the packed tensor (what is computed
+// and the multiplicities: tk_hessian.cu, which serves the other orders).
+//
+// Sums shared between triangles.  With Q = (i, b) (m = 4) and x = w K_{ibcd} the
+// three kinds of contribution are
+//   (A) Hk[c][d] += a_i a_b x        (B) Hk[i][j] += a_b v_ib[j], Hk[b][j] += a_i v_ib[j]
+//   (C) Hk[i][b] += tau_ib           (each with its transpose),
+// v_ib[j] the products of the triangle's symmetric matrix with a, tau_ib its
+// quadratic form.  For a fixed place (c, d) of the triangle let
+//   T_i = sum_b a_b x   and   R_b = sum_i a_i x:
+// then (A) is sum_i a_i T_i, the i-row of (B) the product of the matrix T_i with a
+// and its b-row that of R_b.  So nothing of (B) is done per triangle: a warp
+// that owns 8 x 32 places, NI values of i and a run of b keeps T_i in registers
+// to the end of the run and forms the products of R_b once per b for all its i.
+// Per entry that leaves a load and three multiply-adds (T, R, and the column
+// sums that give tau and R_b's column product).
+//
+// Everything is added into one FP64 matrix Z by atomic adds (Hk = w (Z + Z^T), the
+// second kernel): per b one product with R_b (32 + 8 values), NI values tau,
+// at the end of a run the products with T_i and the places themselves.  Only
+// the order of these FP64 additions differs from call to call.
+//
+// GB300 mapping.  Rows are counted from the last one (c = n-1-8q-r) and columns
+// from the last one (d = n-1-32k-lane), so that only the tiles that the diagonal
+// crosses are masked.  The distance between two rows of a triangle does not
+// depend on b, nor the distance between the slabs of two i: an address is
+// slab(i) + o(b) - D_r, one 32-bit subtraction and a widening multiply-add away.
+// The 8 warps of a block take neighbouring column chunks of the same rows, so a
+// row segment's shared cache lines are read from HBM once (1.39 GB for 1.38).
+//
+// What bounds it (m = 4, n = 300 FP32): the instructions, some 540 per step of
+// 1024 entries (209 M in all, issue 38 % busy with 16 warps an SM; without the
+// loads it takes the same time, without the atomic additions a tenth less); 128
+// registers hold T (4 i x 8 rows), the loaded entries and R.  0.50 ms against
+// 3.59 for the pass of tk_hessian.cu (947 M instructions, three block barriers
+// per 8 triangles); FP64 4.6 against 20.4 ms (FP64 units); m = 4, n = 400 1.28 ms,
+// n = 120 0.064.  Eight values of i in 255 registers (8 warps an SM) take 0.71 ms,
+// two in 80 (24 warps) 0.56.
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "tk_contract_impl.cuh"
+
+namespace tk {
+
+constexpr int kH34Rows = 8;
+constexpr int kH34MaxQ = TK_MAX_POINTS / kH34Rows;
+
+struct H34Params {
+  int n;
+  int bc;              // values of b per item
+  int nq;              // row blocks
+  const unsigned char *K;
+  const double *alpha;
+  double *Z;
+  int pre[kH34MaxQ + 1];  // items before each row block
+};
+
+// items of row block q: column chunks x (i block, run of b)
+TK_HD int h34_chunks(int q) { return (kH34Rows * q + kH34Rows - 1) / 32 + 1; }
+TK_HD int h34_runs(int nb, int bc) { return (nb + bc - 1) / bc; }
+
+// Sum of V values over the warp's lanes, scattered: lane l ends with the sum of
+// value l / (32 / V) (V = 8 or 16).
+template <int V, typename CT>
+__device__ __forceinline__ CT h34_reduce(CT (&v)[V], int lane) {
+#pragma unroll
+  for (int k = 16, cnt = V / 2; k >= 1; k >>= 1, cnt >>= 1) {
+    if (cnt >= 1) {
+      const bool up = (lane & k) != 0;
+#pragma unroll
+      for (int j = 0; j < V / 2; ++j) {
+        if (j < cnt) {
+          const CT send = up ? v[j] : v[j + cnt];
+          const CT keep = up ? v[j + cnt] : v[j];
+          v[j] = keep + __shfl_xor_sync(0xffffffffu, send, k);
+        }
+      }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], k);
+    }
+  }
+  return v[0];
+}
+
+template <typename ST, typename CT, int M, int NI, int MINB>
+__global__ void __launch_bounds__(256, MINB) hess34_kernel(H34Params p) {
+  constexpr int NR = kH34Rows;
+  extern __shared__ __align__(16) unsigned char h34_smem[];
+  CT *a_s = reinterpret_cast<CT *>(h34_smem);
+  const int n = p.n, lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) a_s[i] = (CT)p.alpha[i];
+  __syncthreads();
+  const int item = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (item >= p.pre[p.nq]) return;
+  int q = 0;
+  {
+    int lo = 0, hi = p.nq - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (p.pre[mid] <= item) lo = mid; else hi = mid - 1;
+    }
+    q = lo;
+  }
+  const int cmax = n - 1 - NR * q, cmin = cmax - (NR - 1);
+  const int nch = h34_chunks(q);
+  int run = (item - p.pre[q]) / nch;
+  const int ch = (item - p.pre[q]) - run * nch;
+  int i0 = 0;
+  if (M == 4) {
+    for (;; i0 += NI) {
+      const int r = h34_runs(cmax + 1 - i0, p.bc);
+      if (run < r) break;
+      run -= r;
+    }
+  }
+  const int b0 = i0 + run * p.bc, b1 = min(b0 + p.bc, cmax + 1);
+  const int d = n - 1 - 32 * ch - lane;
+
+  // the tensor's slab of each i, as if its triangles began at b = 0 (lane ii
+  // finds the ii-th)
+  const ST *slab[NI];
+  CT ai[NI];
+  {
+    const int i = i0 + (lane < NI ? lane : 0);
+    int64_t off = 0;
+    if (M == 4 && i < n) off = multiset(n, 4) - multiset(n - i, 4) - (multiset(n, 3) - multiset(n - i, 3));
+#pragma unroll
+    for (int ii = 0; ii < NI; ++ii) {
+      slab[ii] = reinterpret_cast<const ST *>(p.K) + __shfl_sync(0xffffffffu, off, ii);
+      ai[ii] = M == 3 ? CT(1) : i0 + ii < n ? a_s[i0 + ii] : CT(0);
+    }
+  }
+  CT ac[NR];
+  uint32_t mask = 0, half = 0;  // places of this lane in the triangle; those on the diagonal
+#pragma unroll
+  for (int r = 0; r < NR; ++r) {
+    const int c = cmax - r;
+    ac[r] = c >= 0 ? a_s[c] : CT(0);
+    mask |= (c >= 0 && d >= c) ? 1u << r : 0u;
+    half |= d == c ? 1u << r : 0u;
+  }
+  const CT ad = d >= 0 ? a_s[d] : CT(0);
+  const bool full = __all_sync(0xffffffffu, mask == (1u << NR) - 1 && half == 0);
+  const int dr = NR * q + 1;  // n - cmax
+
+  CT T[NI][NR];
+#pragma unroll
+  for (int ii = 0; ii < NI; ++ii)
+#pragma unroll
+    for (int r = 0; r < NR; ++r) T[ii][r] = CT(0);
+  int s3 = (int)(multiset(n, 3) - multiset(n - b0, 3));  // entries of a slab before its triangle b
+
+  // the entries of the next b are loaded between the sums of the current one
+  // and the warp's reductions
+  CT x[NI][NR];
+  auto load = [&](int b) {
+    const int o0 = s3 + (((cmax - b) * (2 * n - b - cmax + 1)) >> 1) + d - cmax;
+    s3 += ((n - b) * (n - b + 1)) >> 1;
+    const bool inner = b < cmin && (M == 3 || b >= i0 + NI);
+    if (inner && full) {
+#pragma unroll
+      for (int ii = 0; ii < NI; ++ii)
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+          x[ii][r] = ld_elem<ST, CT>(slab[ii] + (o0 - (r * dr + (r * (r - 1)) / 2)));
+    } else if (inner) {
+#pragma unroll
+      for (int ii = 0; ii < NI; ++ii)
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          CT v = CT(0);
+          if (mask >> r & 1) v = ld_elem<ST, CT>(slab[ii] + (o0 - (r * dr + (r * (r - 1)) / 2)));
+          x[ii][r] = (half >> r & 1) ? CT(0.5) * v : v;
+        }
+    } else {
+      // i reaches b, or b the rows: triangles and rows that are not there, and
+      // the multiplicities of i = b and c = b
+#pragma unroll
+      for (int ii = 0; ii < NI; ++ii)
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          const int i = i0 + ii, c = cmax - r;
+          CT v = CT(0);
+          if ((mask >> r & 1) && c >= b && (M == 3 || i <= b))
+            v = ld_elem<ST, CT>(slab[ii] + (o0 - (r * dr + (r * (r - 1)) / 2)));
+          const int kb = (M == 4 && i == b) ? 2 : 1;
+          CT f = (half >> r & 1) ? CT(0.5) : CT(1);
+          if (kb == 2) f *= CT(0.5);
+          if (c == b) {
+            f *= kInvSmall<CT>[kb + 1];
+            if (d == c) f *= CT(2) * kInvSmall<CT>[kb + 2];
+          }
+          x[ii][r] = f * v;
+        }
+    }
+  };
+
+  for (int b = b0 - 1; b < b1; ++b) {
+    // T_i, R_b and, per i, the column sums
+    CT R[NR], red[M == 4 ? NR + NI : NR], col = CT(0);
+    if (b >= b0) {
+      const CT ab = a_s[b];
+#pragma unroll
+      for (int r = 0; r < NR; ++r) R[r] = CT(0);
+#pragma unroll
+      for (int ii = 0; ii < NI; ++ii) {
+        CT cs = CT(0);
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          T[ii][r] = fmx(ab, x[ii][r], T[ii][r]);
+          R[r] = fmx(ai[ii], x[ii][r], R[r]);
+          cs = fmx(ac[r], x[ii][r], cs);
+        }
+        col = fmx(ai[ii], cs, col);
+        if constexpr (M == 4) red[NR + ii] = cs * ad;
+      }
+    }
+    if (b + 1 < b1) load(b + 1);
+    if (b < b0) continue;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) red[r] = R[r] * ad;
+    if (d >= 0) atomicAdd(p.Z + (size_t)b * n + d, (double)col);
+    if constexpr (M == 4 && NI == 8) {
+      const CT s = h34_reduce<16>(red, lane);
+      const int v = lane >> 1;  // row v, or i of value v - 8
+      if ((lane & 1) == 0) {
+        if (v < NR) {
+          if (cmax - v >= 0) atomicAdd(p.Z + (size_t)b * n + (cmax - v), (double)s);
+        } else if (i0 + v - NR <= b) {
+          atomicAdd(p.Z + (size_t)(i0 + v - NR) * n + b, (double)s);
+        }
+      }
+    } else if constexpr (M == 4) {
+      CT lo[8], hi[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        lo[j] = red[j];
+        hi[j] = j < NI ? red[NR + j] : CT(0);
+      }
+      const CT s = h34_reduce<8>(lo, lane), t = h34_reduce<8>(hi, lane);
+      const int v = lane >> 2;
+      if ((lane & 3) == 0 && cmax - v >= 0) atomicAdd(p.Z + (size_t)b * n + (cmax - v), (double)s);
+      if ((lane & 3) == 1 && v < NI && i0 + v <= b) atomicAdd(p.Z + (size_t)(i0 + v) * n + b, (double)t);
+    } else {
+      const CT s = h34_reduce<8>(red, lane);
+      const int v = lane >> 2;
+      if ((lane & 3) == 0 && cmax - v >= 0) atomicAdd(p.Z + (size_t)b * n + (cmax - v), (double)s);
+    }
+  }
+
+  // end of the run: the places, and the products of T_i with a
+#pragma unroll
+  for (int r = 0; r < NR; ++r) {
+    CT s = CT(0);
+#pragma unroll
+    for (int ii = 0; ii < NI; ++ii) s = fmx(ai[ii], T[ii][r], s);
+    if (mask >> r & 1) atomicAdd(p.Z + (size_t)(cmax - r) * n + d, (double)s);
+  }
+  if constexpr (M == 4) {
+#pragma unroll
+    for (int ii = 0; ii < NI; ++ii) {
+      const int i = i0 + ii;
+      CT col = CT(0), red[NR];
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        col = fmx(ac[r], T[ii][r], col);
+        red[r] = T[ii][r] * ad;
+      }
+      const CT s = h34_reduce<NR>(red, lane);
+      const int v = lane >> 2;
+      if (i <= cmax) {
+        if (d >= 0) atomicAdd(p.Z + (size_t)i * n + d, (double)col);
+        if ((lane & 3) == 0 && cmax - v >= 0) atomicAdd(p.Z + (size_t)i * n + (cmax - v), (double)s);
+      }
+    }
+  }
+}
+
+// H = w (Z + Z^T), w = M' / (m (m - 1)) of the general entry
+__global__ void __launch_bounds__(256) hess34_sum(int n, double w, const double *Z, double *H) {
+  __shared__ double t[32][33];
+  const int r0 = 32 * blockIdx.y, s0 = 32 * blockIdx.x, x = threadIdx.x & 31;
+  for (int y = threadIdx.x >> 5; y < 32; y += 8)
+    if (s0 + y < n && r0 + x < n) t[y][x] = Z[(size_t)(s0 + y) * n + r0 + x];
+  __syncthreads();
+  for (int y = threadIdx.x >> 5; y < 32; y += 8)
+    if (r0 + y < n && s0 + x < n) H[(size_t)(r0 + y) * n + s0 + x] = w * (Z[(size_t)(r0 + y) * n + s0 + x] + t[x][y]);
+}
+
+template <typename ST, typename CT, int M, int NI, int MINB>
+static int launch_h34(H34Params &p, int sms, cudaStream_t st) {
+  const int n = p.n;
+  p.nq = (n + kH34Rows - 1) / kH34Rows;
+  // steps (one b of an item) of the whole pass; runs long enough that the work
+  // at their end (some four steps) stays small, short enough for three rounds
+  // of the 16 warps per SM
+  int64_t steps = 0;
+  for (int q = 0; q < p.nq; ++q) {
+    const int nc = n - kH34Rows * q;  // values of b
+    for (int i0 = 0; i0 < (M == 4 ? nc : 1); i0 += NI) steps += (int64_t)h34_chunks(q) * (nc - i0);
+  }
+  const int64_t want = steps / ((int64_t)sms * 48);
+  p.bc = (int)std::max<int64_t>(4, std::min<int64_t>(64, want));
+  int64_t items = 0;
+  for (int q = 0; q < p.nq; ++q) {
+    p.pre[q] = (int)items;
+    const int nc = n - kH34Rows * q;
+    for (int i0 = 0; i0 < (M == 4 ? nc : 1); i0 += NI) items += (int64_t)h34_chunks(q) * h34_runs(nc - i0, p.bc);
+  }
+  p.pre[p.nq] = (int)items;
+  hess34_kernel<ST, CT, M, NI, MINB><<<(unsigned)((items + 7) / 8), 256, n * sizeof(CT), st>>>(p);
+  TK_CUDA_CHECK(cudaGetLastError());
+  return TK_OK;
+}
+
+int hessian34(int m, int n, int storage, const void *K, const double *alpha, double *H, double *Z, cudaStream_t st) {
+  DevInfo di;
+  int rc = dev_info(&di);
+  if (rc != TK_OK) return rc;
+  H34Params p;
+  p.n = n;
+  p.K = reinterpret_cast<const unsigned char *>(K);
+  p.alpha = alpha;
+  p.Z = Z;
+  if (m == 3) {
+    if (storage == TK_F64) rc = launch_h34<double, double, 3, 1, 2>(p, di.sms, st);
+    else if (storage == TK_F32) rc = launch_h34<float, float, 3, 1, 4>(p, di.sms, st);
+    else rc = launch_h34<__nv_bfloat16, float, 3, 1, 4>(p, di.sms, st);
+  } else {
+    if (storage == TK_F64) rc = launch_h34<double, double, 4, 4, 1>(p, di.sms, st);
+    else if (storage == TK_F32) rc = launch_h34<float, float, 4, 4, 2>(p, di.sms, st);
+    else rc = launch_h34<__nv_bfloat16, float, 4, 4, 2>(p, di.sms, st);
+  }
+  if (rc != TK_OK) return rc;
+  const unsigned g = (unsigned)((n + 31) / 32);
+  hess34_sum<<<dim3(g, g), 256, 0, st>>>(n, m == 4 ? 2.0 : 1.0, Z, H);
+  TK_CUDA_CHECK(cudaGetLastError());
+  return TK_OK;
+}
+
+}  // namespace tk

@@ -105,6 +105,8 @@ size_t build_tc_workspace_bytes(int m, int n, int d);
 int build_tc(int m, int n, int d, const double *X, int feat, int degree, int storage, int64_t off_lo, int64_t off_hi,
              void *K, void *work, size_t work_bytes, cudaStream_t st);
 int build_tc_status(cudaStream_t st);
+// Full Hessian pass at orders 3 and 4; Z: n x n zeroed FP64 values.
+int hessian34(int m, int n, int storage, const void *K, const double *alpha, double *H, double *Z, cudaStream_t st);
 extern int g_build_tc_mode;  // 0: where it pays, 1: always (FP32/BF16), -1: never
 extern tk_batched_config g_batched_cfg;
 // resolved batched launch shape; returns false when the kernel does not cover it
