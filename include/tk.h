@@ -110,10 +110,11 @@ int tk_build_packed(int m, int64_t n, int64_t d, const double *X, int feat,
                     int degree, int storage_dtype, void *K, void *stream);
 
 /* Which kernel builds FP32 / BF16 storage: 0 (default) = the tensor-core build
- * (tcgen05.mma kind::f16 over three-part BF16 splits of the operands) for orders
- * m >= 3 beyond the smallest sizes (but not for the exponential map into FP32), 1 =
- * for every build of m >= 3, -1 = the SIMT build.  FP64 storage is built on the
- * FP64 units.  Process-wide. */
+ * (tcgen05.mma kind::f16 over three-part BF16 splits of the operands) for FP32
+ * storage of orders m >= 3 beyond the smallest sizes (but not for the exponential
+ * map), the SIMT build otherwise; 1 = the tensor-core build for every build of
+ * m >= 3; -1 = the SIMT build.  FP64 storage is built on the FP64 units.
+ * Process-wide. */
 int tk_build_set_config(int tensor_cores);
 
 /* Status of the tensor-core builds issued so far on the current device:

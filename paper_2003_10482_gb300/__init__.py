@@ -304,8 +304,8 @@ def tk_umma_probe(A: torch.Tensor, B: torch.Tensor, split: bool = False, stream=
 
 
 def tk_build_set_config(tensor_cores: int = 0) -> None:
-    """Which kernel builds FP32 / BF16 storage: 0 = the tensor-core build where it
-    pays, 1 = always (orders m >= 3), -1 = the SIMT build."""
+    """Which kernel builds FP32 / BF16 storage: 0 = the tensor-core build for FP32
+    where it pays, 1 = always (orders m >= 3), -1 = the SIMT build."""
     _check(lib().tk_build_set_config(int(tensor_cores)))
 
 

@@ -1,7 +1,7 @@
 // Packed build of the order-m tensor kernel (Section 4), stored in the
 // sorted-tuple order of Section 5, on the FP32 and FP64 units; tk_build_tc.cu
-// holds the tensor-core build, which takes FP32 / BF16 storage beyond the
-// smallest sizes (build_uses_tc).
+// holds the tensor-core build, which takes FP32 storage beyond the smallest
+// sizes (build_uses_tc).
 //
 // build_pairs_f64 (FP64 storage, m >= 3) is the matrix product prefixes x pairs
 // of tk_build_tc.cu on the FP64 units.  GB300 does two FP64 multiply-adds per
@@ -10,8 +10,8 @@
 // 64 x 64 tiles per triangle (four fifths of their products outside the
 // triangles), 0.61 ms here, 0.95 of the units' measured 1.06 TFLOP/s.
 //
-// build_kernel (m = 2; FP32 storage under the exponential map; FP32 / BF16 storage of
-// small arrays, or where the tensor cores are switched off): for a triangle Q = (i_1..i_{m-2}) with last value b,
+// build_kernel (m = 2; BF16 storage; FP32 storage of small arrays, under the
+// exponential map, or where the tensor cores are switched off): for a triangle Q = (i_1..i_{m-2}) with last value b,
 // the entries (Q, c, d), b <= c <= d < n, form the upper triangle of the
 // weighted Gram matrix
 //   G^Q = X_{[b:n]} diag(w_Q) X_{[b:n]}^T,   w_Q[k] = prod_{q in Q} x_{q,k},
@@ -321,7 +321,7 @@ static int64_t build_tasks(int m, int64_t n) {
   return total;
 }
 
-// FP32 / BF16 storage goes to the tensor cores from kMinTcStages 16-feature
+// FP32 storage goes to the tensor cores from kMinTcStages 16-feature
 // stages of build_kernel on: that kernel takes some 25 us + 13 ns per stage
 // (m = 4: n = 40, d = 10, 820 stages 37 us; n = 60, d = 30, 3660 stages 70 us), the
 // tensor-core build's three launches 45-50 us at those sizes.
@@ -336,7 +336,7 @@ static bool build_takes_tc(int storage) {
 
 extern "C" int tk_build_path(int64_t d, int storage) {
   (void)d;
-  return build_takes_tc(storage) ? 1 : 0;
+  return build_takes_tc(storage) && (storage == TK_F32 || g_build_tc_mode > 0) ? 1 : 0;
 }
 
 static bool build_uses_tc(int m, int64_t n, int64_t d, int feat, int storage) {
@@ -346,6 +346,10 @@ static bool build_uses_tc(int m, int64_t n, int64_t d, int feat, int storage) {
   // entry (2e-5 at the exponents FP32 can hold): FP32 storage keeps the sums,
   // and so the entries, of the multiply-add build there
   if (feat == TK_FEAT_EXP && storage == TK_F32) return false;
+  // BF16 storage keeps them too: other last bits of the sums would move some 1e-4
+  // of the entries to the neighbouring BF16 value, and every result of a pass over
+  // the tensor by about 5e-5 of itself
+  if (storage == TK_BF16) return false;
   return build_tasks(m, n) * ((d + kKT - 1) / kKT) > kMinTcStages;
 }
 

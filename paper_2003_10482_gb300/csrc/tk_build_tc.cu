@@ -1,4 +1,4 @@
-// Packed build of FP32 / BF16 storage on the 5th-generation tensor cores
+// Packed build of FP32 (on request BF16) storage on the 5th-generation tensor cores
 // (Section 4 tensor kernel, stored in the order of Section 5).
 //
 // The packed array as a matrix product.  Split a sorted tuple into its prefix
