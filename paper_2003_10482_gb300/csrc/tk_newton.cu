@@ -5,14 +5,21 @@
 //
 // Matrices are stored row-major with leading dimension npad = ceil(n/32)*32;
 // held-out points and the padding get identity rows and columns (their step
-// is then -grad = 0).  The factorisation runs panel by panel (32 columns):
-// the diagonal block is factorised by one block per problem, the panel below
-// it solved by one block per 32-row block, and the trailing matrix updated by
-// one block per 32 x 32 tile; each launch covers every problem of the batch
-// (grid y), so one large problem or many small ones both fill the GPU.  A
-// pivot that is not positive (a tensor rounded to FP32 or BF16 can make the
-// form indefinite by more than lambda) marks the problem; the solver then
-// falls back to the steepest-descent direction for it.
+// is then -grad = 0).  The factorisation runs panel by panel (32 columns): one
+// launch factorises the diagonal block and solves the panel below it, one
+// updates the trailing matrix, one block per 32 x 32 tile; each launch covers
+// every problem of the batch (grid y), so one large problem or many small ones
+// both fill the GPU.  A pivot that is not positive (a tensor rounded to FP32 or
+// BF16 can make the form indefinite by more than lambda) marks the problem; the
+// solver then stops it.
+//
+// GB300 does two FP64 multiply-adds per cycle and SM, and a warp instruction
+// costs its 16 cycles however few of its lanes take part.  So the panel gives
+// every lane a row, in registers: the 32 x 32 triangular solve is then 528 full
+// warp instructions (4.4 us) instead of as many from each of 32 warps with one
+// lane at work (130 us), and the diagonal block likewise (10 against 125 us).
+// The blocks of a panel factorise the diagonal block each for themselves, in
+// the time the launch of a kernel of its own would take.
 #include <math.h>
 
 #include "tk_internal.h"
@@ -37,53 +44,64 @@ __global__ void k_form_newton(int m, int n, int npad, const int *idx, const doub
   H[(size_t)j * npad * npad + (size_t)r * npad + c] = v;
 }
 
-// factorise diagonal block k of every problem in place (lower triangle)
-__global__ void __launch_bounds__(kNP * kNP) k_potrf_diag(int npad, int k, double *H, int *bad) {
-  __shared__ double A[kNP][kNP + 1];
-  const int j = blockIdx.x;
-  double *M = H + (size_t)j * npad * npad + (size_t)k * kNP * npad + k * kNP;
-  const int r = threadIdx.x / kNP, c = threadIdx.x % kNP;
-  A[r][c] = M[(size_t)r * npad + c];
-  __syncthreads();
-  for (int p = 0; p < kNP; ++p) {
-    if (threadIdx.x == 0) {
-      double d = A[p][p];
-      if (!(d > 0.0) || !isfinite(d)) {
-        bad[j] = 1;
-        d = 1.0;
-      }
-      A[p][p] = sqrt(d);
-    }
-    __syncthreads();
-    if (c == p && r > p) A[r][p] /= A[p][p];
-    __syncthreads();
-    if (r > p && c > p && c <= r) A[r][c] -= A[r][p] * A[c][p];
-    __syncthreads();
-  }
-  M[(size_t)r * npad + c] = (c <= r) ? A[r][c] : 0.0;
-}
-
-// panel below diagonal block k: X L_kk^T = A_ik for every block row i > k
-__global__ void __launch_bounds__(kNP * kNP) k_trsm_panel(int npad, int k, double *H) {
+// Diagonal block k of every problem (block x = 0, into Ld: 32 x 32 factors by
+// block) and the panel below it, X L_kk^T = A_ik for block row i = k + x > k, in
+// place.  One warp, lane r <-> row r of the block.
+__global__ void __launch_bounds__(kNP) k_panel(int npad, int k, double *H, double *Ld, int *bad) {
   __shared__ double L[kNP][kNP + 1];
-  __shared__ double X[kNP][kNP + 1];
-  const int i = k + 1 + blockIdx.x;
-  const int j = blockIdx.y;
+  __shared__ double rinv[kNP];
+  const int j = blockIdx.y, r = threadIdx.x;
   double *Hb = H + (size_t)j * npad * npad;
-  const int r = threadIdx.x / kNP, c = threadIdx.x % kNP;
-  L[r][c] = Hb[(size_t)(k * kNP + r) * npad + k * kNP + c];
-  X[r][c] = Hb[(size_t)(i * kNP + r) * npad + k * kNP + c];
-  __syncthreads();
-  // row r of X: forward substitution over the 32 columns (thread c == 0 of each row)
-  if (c == 0) {
-    for (int q = 0; q < kNP; ++q) {
-      double s = X[r][q];
-      for (int t = 0; t < q; ++t) s -= X[r][t] * L[q][t];
-      X[r][q] = s / L[q][q];
+  double a[kNP];
+#pragma unroll
+  for (int q = 0; q < kNP; ++q) L[q][r] = Hb[(size_t)(k * kNP + q) * npad + k * kNP + r];
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < kNP; ++c) a[c] = L[r][c];
+  bool neg = false;
+#pragma unroll
+  for (int p = 0; p < kNP; ++p) {
+    double d = __shfl_sync(0xffffffffu, a[p], p);
+    if (!(d > 0.0) || !isfinite(d)) {
+      neg = true;
+      d = 1.0;
     }
+    const double ri = rsqrt(d);
+    a[p] = r == p ? d * ri : a[p] * ri;
+    if (r == p) rinv[p] = ri;
+    // rows above c get values that nothing reads
+#pragma unroll
+    for (int c = p + 1; c < kNP; ++c) a[c] -= a[p] * __shfl_sync(0xffffffffu, a[p], c);
   }
-  __syncthreads();
-  Hb[(size_t)(i * kNP + r) * npad + k * kNP + c] = X[r][c];
+  if (blockIdx.x == 0) {
+    if (neg && r == 0) bad[j] = 1;
+    double *D = Ld + ((size_t)j * (npad / kNP) + k) * kNP * kNP;
+#pragma unroll
+    for (int c = 0; c < kNP; ++c) D[r * kNP + c] = c <= r ? a[c] : 0.0;
+    return;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < kNP; ++c) L[r][c] = a[c];
+  __shared__ double X[kNP][kNP + 1];
+  double *P = Hb + (size_t)(k + blockIdx.x) * kNP * npad + k * kNP;
+#pragma unroll
+  for (int q = 0; q < kNP; ++q) X[q][r] = P[(size_t)q * npad + r];
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < kNP; ++c) a[c] = X[r][c];
+#pragma unroll
+  for (int q = 0; q < kNP; ++q) {
+    a[q] *= rinv[q];
+#pragma unroll
+    for (int c = q + 1; c < kNP; ++c) a[c] -= a[q] * L[c][q];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < kNP; ++c) X[r][c] = a[c];
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < kNP; ++q) P[(size_t)q * npad + r] = X[q][r];
 }
 
 // trailing update: A_il -= L_ik L_lk^T for k < l <= i
@@ -112,36 +130,69 @@ __global__ void __launch_bounds__(kNP * kNP) k_syrk_update(int npad, int k, int 
   Hb[(size_t)(i * kNP + r) * npad + l * kNP + c] -= s;
 }
 
-// p_b = -(L L^T)^{-1} g_b on kept points (zero elsewhere); one block per problem
+// p_b = -(L L^T)^{-1} g_b on kept points (zero elsewhere); one block per
+// problem, block by block of 32 unknowns: one warp solves the diagonal block
+// (lane <-> unknown), then every thread takes its own rows of the rest.
 __global__ void __launch_bounds__(256) k_chol_solve(int n, int npad, const int *idx, const double *Lf,
-                                                    const double *grad, const uint8_t *mask, double *p,
-                                                    double *scratch) {
-  const int j = blockIdx.x;
+                                                    const double *Ld, const double *grad, const uint8_t *mask,
+                                                    double *p) {
+  __shared__ double y[TK_MAX_POINTS];
+  __shared__ double D[kNP][kNP + 1];
+  const int j = blockIdx.x, nb = npad / kNP, tid = threadIdx.x;
   const int b = idx[j];
   const double *L = Lf + (size_t)j * npad * npad;
-  double *y = scratch + (size_t)j * npad;
-  for (int i = threadIdx.x; i < npad; i += blockDim.x) {
+  const double *Dj = Ld + (size_t)j * nb * kNP * kNP;
+  for (int i = tid; i < npad; i += blockDim.x) {
     const bool keep = i < n && (!mask || mask[(size_t)b * n + i]);
     y[i] = keep ? -grad[(size_t)b * n + i] : 0.0;
   }
-  __syncthreads();
-  // L y = -g, column-oriented: y_i final, then eliminate it from the rows below
-  for (int i = 0; i < npad; ++i) {
-    if (threadIdx.x == 0) y[i] /= L[(size_t)i * npad + i];
+  // L y = -g
+  for (int k = 0; k < nb; ++k) {
+    for (int e = tid; e < kNP * kNP; e += blockDim.x) D[e / kNP][e % kNP] = Dj[(size_t)k * kNP * kNP + e];
     __syncthreads();
-    const double yi = y[i];
-    for (int r = i + 1 + threadIdx.x; r < npad; r += blockDim.x) y[r] -= L[(size_t)r * npad + i] * yi;
+    if (tid < kNP) {
+      double v = y[k * kNP + tid];
+      const double ri = 1.0 / D[tid][tid];
+      for (int q = 0; q < kNP; ++q) {
+        const double vq = __shfl_sync(0xffffffffu, v * ri, q);
+        v = tid == q ? vq : tid > q ? v - D[tid][q] * vq : v;
+      }
+      y[k * kNP + tid] = v;
+    }
+    __syncthreads();
+    for (int r = (k + 1) * kNP + tid; r < npad; r += blockDim.x) {
+      const double *Lr = L + (size_t)r * npad + k * kNP;
+      double s = 0.0;
+#pragma unroll 8
+      for (int q = 0; q < kNP; ++q) s += Lr[q] * y[k * kNP + q];
+      y[r] -= s;
+    }
     __syncthreads();
   }
-  // L^T x = y: row i of L^T is column i of L
-  for (int i = npad - 1; i >= 0; --i) {
-    if (threadIdx.x == 0) y[i] /= L[(size_t)i * npad + i];
+  // L^T x = y
+  for (int k = nb - 1; k >= 0; --k) {
+    for (int e = tid; e < kNP * kNP; e += blockDim.x) D[e / kNP][e % kNP] = Dj[(size_t)k * kNP * kNP + e];
     __syncthreads();
-    const double yi = y[i];
-    for (int r = threadIdx.x; r < i; r += blockDim.x) y[r] -= L[(size_t)i * npad + r] * yi;
+    if (tid < kNP) {
+      double v = y[k * kNP + tid];
+      const double ri = 1.0 / D[tid][tid];
+      for (int q = kNP - 1; q >= 0; --q) {
+        const double vq = __shfl_sync(0xffffffffu, v * ri, q);
+        v = tid == q ? vq : tid < q ? v - D[q][tid] * vq : v;
+      }
+      y[k * kNP + tid] = v;
+    }
+    __syncthreads();
+    for (int c = tid; c < k * kNP; c += blockDim.x) {
+      const double *Lc = L + (size_t)(k * kNP) * npad + c;
+      double s = 0.0;
+#pragma unroll 8
+      for (int q = 0; q < kNP; ++q) s += Lc[(size_t)q * npad] * y[k * kNP + q];
+      y[c] -= s;
+    }
     __syncthreads();
   }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+  for (int i = tid; i < n; i += blockDim.x) {
     const bool keep = !mask || mask[(size_t)b * n + i];
     p[(size_t)b * n + i] = keep ? y[i] : 0.0;
   }
@@ -220,9 +271,10 @@ int take_hessians(int64_t B, int n, const double *flag_dev, const double *Hsrc, 
   return TK_OK;
 }
 
+// Newton matrices, the factors of their diagonal blocks, the flags
 size_t newton_ws_bytes(int n, int64_t nb) {
   const int npad = (n + kNP - 1) / kNP * kNP;
-  return (size_t)nb * ((size_t)npad * npad + npad) * sizeof(double) + (size_t)nb * 2 * sizeof(int);
+  return (size_t)nb * ((size_t)npad * npad + (size_t)npad * kNP) * sizeof(double) + (size_t)nb * 2 * sizeof(int);
 }
 
 // Newton directions of the problems idx[0..nb-1]: Hk holds K[a_b^{m-2}] of
@@ -235,22 +287,21 @@ int newton_directions(int m, int n, int nb, const int *idx_dev, const double *Hk
   const int nbk = npad / kNP;
   unsigned char *w = reinterpret_cast<unsigned char *>(ws);
   double *H = reinterpret_cast<double *>(w);
-  double *y = H + (size_t)nb * npad * npad;
-  int *bad = reinterpret_cast<int *>(y + (size_t)nb * npad);
+  double *Ld = H + (size_t)nb * npad * npad;
+  int *bad = reinterpret_cast<int *>(Ld + (size_t)nb * npad * kNP);
   TK_CUDA_CHECK(cudaMemsetAsync(bad, 0, (size_t)nb * sizeof(int), st));
   dim3 gf((unsigned)((npad + 127) / 128), (unsigned)npad, (unsigned)nb);
   k_form_newton<<<gf, 128, 0, st>>>(m, n, npad, idx_dev, Hk, lambda, mask, H);
   TK_CUDA_CHECK(cudaGetLastError());
   for (int k = 0; k < nbk; ++k) {
-    k_potrf_diag<<<nb, kNP * kNP, 0, st>>>(npad, k, H, bad);
     const int below = nbk - k - 1;
+    k_panel<<<dim3((unsigned)(below + 1), (unsigned)nb), kNP, 0, st>>>(npad, k, H, Ld, bad);
     if (below > 0) {
-      k_trsm_panel<<<dim3((unsigned)below, (unsigned)nb), kNP * kNP, 0, st>>>(npad, k, H);
       k_syrk_update<<<dim3((unsigned)(below * (below + 1) / 2), (unsigned)nb), kNP * kNP, 0, st>>>(npad, k, nbk, H);
     }
   }
   TK_CUDA_CHECK(cudaGetLastError());
-  k_chol_solve<<<nb, 256, 0, st>>>(n, npad, idx_dev, H, grad, mask, p, y);
+  k_chol_solve<<<nb, 256, 0, st>>>(n, npad, idx_dev, H, Ld, grad, mask, p);
   TK_CUDA_CHECK(cudaGetLastError());
   TK_CUDA_CHECK(cudaMemcpyAsync(bad_host, bad, (size_t)nb * sizeof(int), cudaMemcpyDeviceToHost, st));
   TK_CUDA_CHECK(cudaStreamSynchronize(st));
