@@ -31,6 +31,8 @@ tk_contract_config g_contract_cfg = {0, 0, 0, 0, 0, 0, 0, 0};
 
 static const int kMaxWarps = 16;
 
+static const int64_t kMinWarpEntries = 96, kMinPieceEntries = 2048;
+
 static const int kMaxPiecesPerWarp = 16;
 size_t contract_plan_bytes(int sms) { return (size_t)kMaxPiecesPerWarp * 2 * sms * kMaxWarps * sizeof(WarpPlan); }
 size_t contract_part_bytes(int n, int grid) { return (size_t)grid * 2 * (size_t)(n + 2) * sizeof(double); }
@@ -219,7 +221,17 @@ static int resolve(int m, int n, int storage, bool dual, Resolved *r) {
   const int smem_budget = (di.smem_optin - 4096) / r->cps;
   // a buffer holds one full row (n entries) plus the alignment slack of its copy
   const int min_buf = (n * es + 32 + 127) & ~127;
-  int warps = o.warps > 0 ? o.warps : kMaxWarps;
+  // Small tensors get fewer warps and pieces (of the whole tensor's entries, so
+  // that shards of it keep its cut): a piece costs its plan record, its copies'
+  // latency and a flush however few entries it holds.  At least kMinWarpEntries
+  // per warp and kMinPieceEntries per piece: m = 4 n = 40 FP64 72.7 -> 27.4 us
+  // against 16 warps of 16 pieces, n = 60 FP32 62 -> 25, n = 100 71 -> 40, n = 150
+  // 91 -> 67 (16 pieces again from n = 280 on)
+  // (any launch parameter set by the caller keeps the full cut).
+  const bool own = o.warps | o.block_bytes | o.nbuf | o.ctas_per_sm | o.row_cost | o.tri_cost | o.pieces_per_warp | o.schedule;
+  const int64_t entries = own ? INT64_MAX : multiset(n, m), blocks = (int64_t)di.sms * r->cps;
+  int warps = o.warps > 0 ? o.warps
+                          : (int)std::max<int64_t>(4, std::min<int64_t>(kMaxWarps, entries / (blocks * kMinWarpEntries)));
   warps = std::min(warps, max_threads_est(cts, dual, r->nc) / 32);
   int buf = 0;
   for (; warps >= 1; --warps) {
@@ -246,7 +258,9 @@ static int resolve(int m, int n, int storage, bool dual, Resolved *r) {
   const bool cheap_rows = dual || storage == TK_BF16 || m >= 5;
   r->row_cost = o.row_cost > 0 ? o.row_cost : (cheap_rows ? 64 : 256);
   r->tri_cost = o.tri_cost > 0 ? o.tri_cost : (cheap_rows ? 4096 : 4 * r->row_cost);
-  r->ppw = o.pieces_per_warp > 0 ? o.pieces_per_warp : 16;
+  r->ppw = o.pieces_per_warp > 0
+               ? o.pieces_per_warp
+               : (int)std::max<int64_t>(1, std::min<int64_t>(16, entries / (blocks * warps * kMinPieceEntries)));
   if (r->ppw > kMaxPiecesPerWarp) return fail(TK_EINVAL, "pieces_per_warp above %d", kMaxPiecesPerWarp);
   r->schedule = o.schedule > 0 ? o.schedule : 1;
   if (r->schedule > 2) return fail(TK_EINVAL, "schedule must be 1 or 2");
