@@ -170,8 +170,8 @@ size_t tk_contract_workspace_size(int m, int64_t n, int64_t B);
  * Arithmetic: FP64 for TK_F64 storage; FP32 for TK_F32 / TK_BF16 storage with
  * the cross-block reduction and S in FP64.  Each packed entry is read from
  * HBM once per pass.  For TK_F32 / TK_BF16 storage and B at least the
- * batched configuration's min_batch (by default 28, or 16 for r = m-2; see
- * tk_batched_config) one launch serves the whole batch (each entry read once
+ * batched configuration's min_batch (by default at most 28, or 16 for r = m-2;
+ * see tk_batched_config) one launch serves the whole batch (each entry read once
  * for all B vectors, 2B multiply-adds per entry; 4B for r = m-2); otherwise
  * the single-vector pass runs once per b.  Asynchronous; errors that only the
  * device can see (a bounded wait that ran out) are recorded in `work` and
@@ -233,12 +233,16 @@ int tk_contract_get_config(int m, int64_t n, int storage_dtype, int dual, tk_con
  *   slice_mult   blocks per group of vectors = slice_mult * SMs / groups (1 or 2)
  *   min_batch    smallest B that takes the batched kernel (below it the
  *                single-vector pass runs once per vector); 0 = 28 (16 for
- *                r = m-2); a value sets both
+ *                r = m-2), or n/12 (n/16) where the FP32 rows pass serves
+ *                the call and that is less; a value sets both
  *   tensor_cores the tensor-core pass for r = m-1 (tcgen05.mma, TF32 with a
  *                3-term split; the whole tensor, FP32 or BF16 storage,
- *                n <= 320): 0 = where it pays (m = 3 or 4, n >= 64, B >= 128),
- *                1 = wherever it covers the call, -1 = never.  In the result of
- *                tk_batched_get_config: 1 when the call would take it, else 0 */
+ *                n <= 320): 0 = where it pays (m = 3 or 4, n >= 64, B >= 64),
+ *                1 = wherever it covers the call, -1 = never, and neither the
+ *                FP32 rows pass that serves the other batches (and r = m-2) of
+ *                m = 3 and 4, 40 <= n <= 320.  In the result of
+ *                tk_batched_get_config: 1 when the call would take it, else 0.
+ * The first four fields concern the batches that neither of the two serves. */
 typedef struct {
     int vpl;
     int block_bytes;

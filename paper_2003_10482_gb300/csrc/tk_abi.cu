@@ -136,6 +136,8 @@ size_t tk_contract_workspace_size(int m, int64_t n, int64_t B) {
   if (B > 1) need = std::max(need, batched_workspace_bytes((int)n, B, di.sms));
   // room for the tensor-core pass wherever the configuration may take it
   if (tc_covers(m, (int)n, TK_F32, false, B, 0, multiset(n, m))) need = std::max(need, tc_workspace_bytes(m, (int)n, B, di.sms));
+  if (B > 1 && rows_covers(m, (int)n, TK_F32, false, B, 0, multiset(n, m)))
+    need = std::max(need, rows_workspace_bytes(m, (int)n, B, di.sms));
   return need;
 }
 
@@ -171,7 +173,8 @@ static int contract_impl(int m, int64_t n, int storage, const void *K, int64_t o
   // for one vector as for 64 (32 for the HVP), while the single-vector kernel
   // runs at the HBM rate (measured on GB300, m = 4, n = 300: the batched
   // kernel wins from B = 28 for K[a^{m-1}] and from B = 16 for the HVP).
-  if (B >= batched_min_batch(r == m - 2) && storage != TK_F64) {
+  if ((B >= batched_min_batch(r == m - 2) || rows_pays(m, (int)n, storage, r == m - 2, B, off_lo, off_hi)) &&
+      storage != TK_F64) {
     BatchedArgs ba;
     memset(&ba, 0, sizeof(ba));
     ba.m = m;
@@ -190,6 +193,10 @@ static int contract_impl(int m, int64_t n, int storage, const void *K, int64_t o
     ba.work_bytes = work_bytes;
     if (tc_covers(m, (int)n, storage, r == m - 2, B, off_lo, off_hi)) {
       rc = contract_batched_tc(ba, st);
+      if (rc != TK_EUNSUPPORTED) return rc;
+    }
+    if (rows_covers(m, (int)n, storage, r == m - 2, B, off_lo, off_hi)) {
+      rc = contract_batched_rows(ba, st);
       if (rc != TK_EUNSUPPORTED) return rc;
     }
     rc = contract_batched(ba, st);

@@ -1,0 +1,332 @@
+// Batched contraction and Hessian-vector product on the FP32 units, triangle by
+// triangle as a matrix product (included by tk_batched_tc.cu, whose jobs,
+// triangle records and job ranges it shares).
+//
+// As in tk_tc_math.h the row dots Rf_c = sum_d S~_Q[c][d] a_d of all vectors form
+// one product; here S~_Q's rows are gathered into shared memory and multiplied
+// by plain FP32 multiply-adds, so that the result has the accuracy of the other
+// FP32 kernels.  The Hessian-vector product (DUAL) is the derivative along v of
+// the same sums: a block's columns hold the vectors a and, in the other half, the
+// directions v, the product gives Rf(a) and Rf(v), and the epilogue carries dual
+// numbers:
+//   g'_c += (M'/m) (A_Q' Rf_c(a) + A_Q Rf_c(v)),
+//   P' = sum_{c > b} v_c Rf_c(a) + a_c Rf_c(v),  r_b' = Rf_b(v) - h_b v_b/(kb+1),
+// and T, T_rest of tk_tc_math.h by the product rule.
+//
+// GB300 mapping.  A block of 256 threads holds its NC columns of all points in
+// shared memory for the whole pass and walks a range of jobs (up to 96 rows of one
+// triangle).  Per 32-column chunk of d the threads gather 96 x 32 entries (the
+// next chunk's loads are issued before the current chunk's products) and each
+// forms 6 rows x NC/16 columns, the same problems in both halves.  g is added in
+// FP32 to a scratch of the block's own (L2) and from there to FP64 every
+// kRowsFlushJobs jobs.
+#pragma once
+
+namespace tk {
+
+constexpr int kRgThreads = 256;
+constexpr int kRgPitch = tc::kRowsPerJob + 2;  // words per column of a gathered chunk (8-byte aligned rows, 2-way stores)
+constexpr int kRgFlushJobs = 64;
+
+struct RgParams {
+  TcParams t;      // jobs, tris, range, P, at (n x Bpad), gpart, spart as in the tensor-core pass
+  float *g32;      // [block][n16][problems per slice]
+};
+
+template <int NC>
+constexpr size_t rg_smem(int nkc) {
+  return (size_t)(32 * nkc * NC + 2 * 32 * kRgPitch + 16 * NC + 2 * NC) * sizeof(float);
+}
+
+// the chunk's 12 values of a thread: those of stage_rows, unsplit
+template <typename ST>
+__device__ __forceinline__ void rg_load(const TcParams &p, const TcTri &tri, int cs, int npad, int d0, int t,
+                                        float (&x)[3][4]) {
+  const int n = p.n, b = tri.b, bb = b < 0 ? 0 : b;
+  const int span = 2 * n - bb + 1;
+  const ST *__restrict__ Kt = reinterpret_cast<const ST *>(p.K) + tri.base;
+#pragma unroll
+  for (int sb = 0; sb < 3; ++sb) {
+    const int jb = 32 * sb;
+    const bool lower = d0 + 31 < cs + jb;   // every column below every row of the sub-block
+    const bool upper = d0 >= cs + jb + 31;  // every column at or above every row
+    const int j = lower ? jb + (t & 31) : jb + (t >> 3);
+    const int k4 = lower ? 4 * (t >> 5) : 4 * (t & 7);
+    const int c = cs + j, d = d0 + k4;
+    if (lower) {
+      int off = (((d - bb) * (span - d)) >> 1) + (c - d);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const bool ok = j < npad && d + e >= bb && c < n;
+        x[sb][e] = ok ? ld_elem<ST, float>(Kt + off) : 0.f;
+        off += n - d - e - 1;
+      }
+    } else if (upper) {
+      const int off = (((c - bb) * (span - c)) >> 1) + (d - c);
+      const bool okr = j < npad && c >= bb;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[sb][e] = (okr && d + e < n) ? ld_elem<ST, float>(Kt + off + e) : 0.f;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int de = d + e;
+        const int r = min(c, de), s2 = max(c, de);
+        const bool ok = j < npad && r >= bb && s2 < n;
+        const int off = (((r - bb) * (span - r)) >> 1) + (s2 - r);
+        x[sb][e] = ok ? ld_elem<ST, float>(Kt + off) : 0.f;
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ void rg_store(const TcTri &tri, int cs, int npad, int d0, int t, const float (&x)[3][4],
+                                         float *buf) {
+  const float fb = kInvSmall<float>[tri.kb + 1];
+#pragma unroll
+  for (int sb = 0; sb < 3; ++sb) {
+    const int jb = 32 * sb;
+    if (jb >= npad) break;
+    const bool lower = d0 + 31 < cs + jb;
+    const int j = lower ? jb + (t & 31) : jb + (t >> 3);
+    const int k4 = lower ? 4 * (t >> 5) : 4 * (t & 7);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) buf[(k4 + e) * kRgPitch + j] = d0 + k4 + e == tri.b ? x[sb][e] * fb : x[sb][e];
+  }
+}
+
+template <typename ST, bool DUAL, int NC>
+__global__ void __launch_bounds__(kRgThreads, 1) rows_batched_kernel(RgParams rp) {
+  constexpr int H = NC / 2;        // columns of a half
+  constexpr int CW = H / 16;       // a thread's columns of each half
+  constexpr int NP = DUAL ? H : NC;  // problems of the slice
+  const TcParams &p = rp.t;
+  extern __shared__ __align__(16) float rg_sm[];
+  if (plan_is_stale(p.status, p.m, p.n, p.P, -2, -2)) return;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, w = tid >> 5;
+  const int n = p.n, nrow = 32 * p.nkc;
+  const int slice = blockIdx.x / p.P, part = blockIdx.x % p.P;
+  const int j_lo = p.range[part], j_hi = p.range[part + 1];
+  float *X = rg_sm;                        // [nrow][NC]
+  float *buf = X + (size_t)nrow * NC;      // [2][32][kRgPitch]
+  float *red = buf + 2 * 32 * kRgPitch;    // [16][NC]
+  float *rfb = red + 16 * NC;              // [NC] (and NC spare)
+  for (int i = tid; i < nrow * NC; i += kRgThreads)
+    X[i] = i / NC < n ? p.at[(size_t)(i / NC) * p.Bpad + (size_t)slice * NC + i % NC] : 0.f;
+  double *gp = p.gpart + (size_t)blockIdx.x * p.n16 * kTcSlice;
+  float *g32 = rp.g32 + (size_t)blockIdx.x * p.n16 * NP;
+  for (int i = tid; i < n * NP; i += kRgThreads) {
+    gp[(size_t)(i / NP) * kTcSlice + i % NP] = 0.0;
+    g32[i] = 0.f;
+  }
+  for (int i = tid; i < NC; i += kRgThreads) rfb[i] = 0.f;
+  __syncthreads();
+  const float inv_m = 1.f / (float)p.m;
+  double S64 = 0.0;
+  float P1[2 * CW];  // DUAL: P and P' of CW problems, else P of 2 CW problems
+#pragma unroll
+  for (int j = 0; j < 2 * CW; ++j) P1[j] = 0.f;
+  int since_flush = 0;
+  auto flush = [&]() {
+    for (int i = tid; i < n * NP; i += kRgThreads) {
+      gp[(size_t)(i / NP) * kTcSlice + i % NP] += (double)g32[i];
+      g32[i] = 0.f;
+    }
+  };
+
+  for (int jx = j_lo; jx < j_hi; ++jx) {
+    const TcJob job = p.jobs[jx];
+    const TcTri tri = p.tris[job.tri];
+    const int b = tri.b, cs = job.cs, npad = job.npad;
+    float acc[6][2 * CW];
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+#pragma unroll
+      for (int j = 0; j < 2 * CW; ++j) acc[i][j] = 0.f;
+    float x[3][4];
+    rg_load<ST>(p, tri, cs, npad, 32 * job.kc0, tid, x);
+    rg_store(tri, cs, npad, 32 * job.kc0, tid, x, buf);
+    __syncthreads();
+    const bool mine = 12 * w < npad;  // the warp's 12 rows are among the job's
+    for (int kc = job.kc0; kc < p.nkc; ++kc) {
+      const bool more = kc + 1 < p.nkc;
+      if (more) rg_load<ST>(p, tri, cs, npad, 32 * (kc + 1), tid, x);
+      if (mine) {
+        const float *sp = buf + ((kc - job.kc0) & 1) * 32 * kRgPitch + 6 * ty;
+        const float *xp = X + (size_t)32 * kc * NC + CW * tx;
+#pragma unroll 8
+        for (int k = 0; k < 32; ++k) {
+          float s[6], xv[2 * CW];
+#pragma unroll
+          for (int i = 0; i < 6; i += 2) {
+            const float2 f = *reinterpret_cast<const float2 *>(sp + k * kRgPitch + i);
+            s[i] = f.x;
+            s[i + 1] = f.y;
+          }
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if constexpr (CW == 4) {
+              const float4 f = *reinterpret_cast<const float4 *>(xp + k * NC + H * h);
+              xv[4 * h] = f.x;
+              xv[4 * h + 1] = f.y;
+              xv[4 * h + 2] = f.z;
+              xv[4 * h + 3] = f.w;
+            } else {
+              const float2 f = *reinterpret_cast<const float2 *>(xp + k * NC + H * h);
+              xv[2 * h] = f.x;
+              xv[2 * h + 1] = f.y;
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < 6; ++i)
+#pragma unroll
+            for (int j = 0; j < 2 * CW; ++j) acc[i][j] = __fmaf_rn(s[i], xv[j], acc[i][j]);
+        }
+      }
+      if (more) rg_store(tri, cs, npad, 32 * (kc + 1), tid, x, buf + ((kc + 1 - job.kc0) & 1) * 32 * kRgPitch);
+      __syncthreads();
+    }
+
+    // ---- rows: g, and the triangle's quadratic-form sums
+    float coef[2 * CW];  // DUAL: (M'/m) A_Q', then (M'/m) A_Q; else (M'/m) A_Q
+    const float mm = (float)tri.mprime * inv_m;
+#pragma unroll
+    for (int j = 0; j < CW; ++j) {
+      if constexpr (DUAL) {
+        float A = 1.f, Ad = 0.f;
+        for (int q = 0; q < tri.nq; ++q) {
+          const float a = X[(size_t)tri.q[q] * NC + CW * tx + j], v = X[(size_t)tri.q[q] * NC + H + CW * tx + j];
+          Ad = Ad * a + A * v;
+          A *= a;
+        }
+        coef[j] = mm * Ad;
+        coef[CW + j] = mm * A;
+      } else {
+        float A0 = 1.f, A1 = 1.f;
+        for (int q = 0; q < tri.nq; ++q) {
+          A0 *= X[(size_t)tri.q[q] * NC + CW * tx + j];
+          A1 *= X[(size_t)tri.q[q] * NC + H + CW * tx + j];
+        }
+        coef[j] = mm * A0;
+        coef[CW + j] = mm * A1;
+      }
+    }
+    if (mine) {
+#pragma unroll
+      for (int i = 0; i < 6; ++i) {
+        const int r = 6 * ty + i, c = cs + r;
+        if (r >= npad || c < b || c >= n) continue;
+        const float *xc = X + (size_t)c * NC + CW * tx;
+        float *g = g32 + (size_t)c * NP + CW * tx;
+#pragma unroll
+        for (int j = 0; j < CW; ++j) {
+          const float Ra = acc[i][j], Rv = acc[i][CW + j];
+          if constexpr (DUAL) {
+            g[j] += coef[j] * Ra + coef[CW + j] * Rv;
+            if (c > b) {
+              P1[j] += xc[j] * Ra;
+              P1[CW + j] += xc[H + j] * Ra + xc[j] * Rv;
+            }
+          } else {
+            g[j] += coef[j] * Ra;
+            g[H + j] += coef[CW + j] * Rv;
+            if (c > b) {
+              P1[j] += xc[j] * Ra;
+              P1[CW + j] += xc[H + j] * Rv;
+            }
+          }
+          if (c == b) {
+            rfb[CW * tx + j] = Ra;
+            rfb[H + CW * tx + j] = Rv;
+          }
+        }
+      }
+    }
+    if (job.flags & 2) {
+      // ---- the triangle's last job: its prefix-value terms (and S)
+#pragma unroll
+      for (int j = 0; j < CW; ++j) {
+        red[ty * NC + CW * tx + j] = P1[j];
+        red[ty * NC + H + CW * tx + j] = P1[CW + j];
+        P1[j] = P1[CW + j] = 0.f;
+      }
+      __syncthreads();
+      if (tid < NP) {
+        float P = 0.f, Pd = 0.f;
+        for (int r = 0; r < 16; ++r) {
+          P += red[r * NC + tid];
+          if (DUAL) Pd += red[r * NC + H + tid];
+        }
+        const float hb = b >= 0 ? ld_entry<ST>(p.K, tri.base) : 0.f;
+        const float ab = b >= 0 ? X[(size_t)b * NC + tid] : 0.f;
+        float T, Tr, Td = 0.f, Trd = 0.f;
+        tc::finish_triangle<float>(b, tri.kb, (float)tri.mprime, P, rfb[tid], hb, ab, &T, &Tr);
+        if constexpr (DUAL) {
+          const float hm = 0.5f * (float)tri.mprime;
+          if (b < 0) {
+            Td = Trd = hm * Pd;
+          } else {
+            const float k1 = kInvSmall<float>[tri.kb + 1], k2 = kInvSmall<float>[tri.kb + 2];
+            const float vb = X[(size_t)b * NC + H + tid];
+            const float rb = rfb[tid] - hb * ab * k1, rbd = rfb[H + tid] - hb * vb * k1;
+            Trd = hm * (Pd - (vb * rb + ab * rbd) * k1);
+            Td = Trd + (float)tri.mprime * k1 * (vb * (rb + hb * ab * k2) + ab * (rbd + hb * vb * k2));
+          }
+        }
+        float AQ = 1.f;
+        for (int q = 0; q < tri.nq; ++q) AQ *= X[(size_t)tri.q[q] * NC + tid];
+        if (!DUAL) S64 += (double)(AQ * T);
+        for (int q = 0; q < tri.nq; ++q) {
+          if (q > 0 && tri.q[q] == tri.q[q - 1]) continue;
+          const int l = tri.q[q];
+          int cnt = 0;
+          float B = 1.f, Bd = 0.f;
+          bool skipped = false;
+          for (int qq = 0; qq < tri.nq; ++qq) {
+            if (tri.q[qq] == l) {
+              ++cnt;
+              if (!skipped) {
+                skipped = true;
+                continue;
+              }
+            }
+            const float a = X[(size_t)tri.q[qq] * NC + tid];
+            if (DUAL) Bd = Bd * a + B * X[(size_t)tri.q[qq] * NC + H + tid];
+            B *= a;
+          }
+          const float f = (float)cnt * inv_m;
+          g32[(size_t)l * NP + tid] += DUAL ? f * (Bd * (l == b ? Tr : T) + B * (l == b ? Trd : Td))
+                                            : f * B * (l == b ? Tr : T);
+        }
+      }
+      __syncthreads();
+    }
+    if (++since_flush == kRgFlushJobs) {
+      __syncthreads();
+      flush();
+      __syncthreads();
+      since_flush = 0;
+    }
+  }
+  __syncthreads();
+  flush();
+  if (!DUAL && tid < NP) p.spart[(size_t)blockIdx.x * kTcSlice + tid] = S64;
+}
+
+// at[d][slot]: column slot of slice s is problem s NP + slot (its direction in the
+// other half when V is given)
+__global__ void rows_prep_vectors(int n, int64_t B, int Bpad, int NC, int NP, int vec_dtype, const void *A,
+                                  const void *V, float *at) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (int64_t)Bpad * n) return;
+  const int slot = (int)(i / n), d = (int)(i % n);
+  const int in = slot % NC;
+  const int64_t b = (int64_t)(slot / NC) * NP + in % NP;
+  const void *src = in < NP ? A : V;
+  float x = 0.f;
+  if (b < B)
+    x = vec_dtype == TK_F64 ? (float)reinterpret_cast<const double *>(src)[(size_t)b * n + d]
+                            : reinterpret_cast<const float *>(src)[(size_t)b * n + d];
+  at[(size_t)d * Bpad + slot] = x;
+}
+
+}  // namespace tk

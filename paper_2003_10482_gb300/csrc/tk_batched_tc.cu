@@ -54,6 +54,7 @@ constexpr int kTcGatherThreads = 32 * kTcGatherWarps;
 constexpr int kTcThreads = 32 * (kTcEpiWarps + kTcGatherWarps + 1);  // + warp 12: issues the MMAs
 constexpr int kTcSlice = 128;        // vectors per block (M of the MMA)
 constexpr int kTcMaxN = 320;         // g accumulator columns left beside the two job accumulators
+constexpr int kRgMinN = 40;          // points from which the FP32 rows pass is taken
 constexpr int kTcFlushJobs = 128;    // jobs between FP64 flushes of the g accumulator
 constexpr uint32_t kTcAccCols = 96;  // tensor-memory columns: [0, 96) and [96, 192) the two job accumulators,
 constexpr uint32_t kTcAColsG = 192;  // [192, 192 + n16) the g accumulator
@@ -187,6 +188,10 @@ __device__ __forceinline__ void stage_rows(const TcParams &p, const TcTri &tri, 
     *reinterpret_cast<float4 *>(blo + so) = make_float4(l[0], l[1], l[2], l[3]);
   }
 }
+
+}  // namespace tk
+#include "tk_batched_rows.cuh"
+namespace tk {
 
 // Bounded wait on an mbarrier phase; once any wait of the block has run out
 // every later wait returns false at once, so all roles leave their loops.
@@ -443,16 +448,17 @@ __global__ void tc_prep_vectors(int n, int nkc, int64_t B, int Bpad, int vec_dty
   if (d < n) at[(size_t)d * Bpad + beta] = x;
 }
 
-// G[b][c] and S[b]: the blocks' partials of b's slice, summed in a fixed order.
-__global__ void tc_reduce(int m, int n, int n16, int64_t B, int P, const double *gpart, const double *spart,
-                          int out_dtype, void *G, double *S, const int *status) {
+// G[b][c] and S[b]: the blocks' partials of b's slice (np problems each), summed
+// in a fixed order and scaled.
+__global__ void tc_reduce(int m, int n, int n16, int64_t B, int np, double scale, int P, const double *gpart,
+                          const double *spart, int out_dtype, void *G, double *S, const int *status) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t b = blockIdx.y;
   if (c > n || (c == n && !S)) return;
   const volatile WsHeader *wh = reinterpret_cast<const volatile WsHeader *>(status);
   if (!(wh->plan_m == m && wh->plan_n == n && wh->plan_pieces == P && wh->plan_lo == -2 && wh->plan_hi == -2))
     return;
-  const int slice = (int)(b / kTcSlice), bl = (int)(b % kTcSlice);
+  const int slice = (int)(b / np), bl = (int)(b % np);
   double s = 0.0;
   if (c == n) {
     for (int k = 0; k < P; ++k) s += spart[(size_t)(slice * P + k) * kTcSlice + bl];
@@ -460,6 +466,7 @@ __global__ void tc_reduce(int m, int n, int n16, int64_t B, int P, const double 
     return;
   }
   for (int k = 0; k < P; ++k) s += gpart[((size_t)(slice * P + k) * n16 + c) * kTcSlice + bl];
+  s *= scale;
   if (out_dtype == TK_F64) reinterpret_cast<double *>(G)[b * n + c] = s;
   else reinterpret_cast<float *>(G)[b * n + c] = (float)s;
 }
@@ -629,6 +636,40 @@ size_t tc_workspace_bytes(int m, int n, int64_t B, int sms) {
   return tc_layout(n, B, sms, nj, nt).total;
 }
 
+// Make sure the workspace holds the jobs, triangles and job ranges of (m, n, P).
+static int tc_upload_plan(int m, int n, int P, size_t njobs, size_t ntris, const TcLayout &L, void *work,
+                          cudaStream_t st) {
+  unsigned char *ws = reinterpret_cast<unsigned char *>(work);
+  int dev = 0;
+  TK_CUDA_CHECK(cudaGetDevice(&dev));
+  {
+    std::lock_guard<std::mutex> lk(g_tcmu);
+    TcKey key{m, n, P};
+    auto up = g_tcup.find({dev, work});
+    if (up != g_tcup.end() && !(up->second < key) && !(key < up->second)) return TK_OK;
+    const TcPlan &pl = tc_plan_for(m, n, P);
+    if (pl.jobs.size() != njobs || pl.tris.size() != ntris)
+      return fail(TK_EINVAL, "tensor-core plan: %zu jobs / %zu triangles, layout sized for %zu / %zu",
+                  pl.jobs.size(), pl.tris.size(), njobs, ntris);
+    TK_CUDA_CHECK(cudaMemcpyAsync(ws + L.jobs, pl.jobs.data(), pl.jobs.size() * sizeof(TcJob),
+                                  cudaMemcpyHostToDevice, st));
+    TK_CUDA_CHECK(cudaMemcpyAsync(ws + L.tris, pl.tris.data(), pl.tris.size() * sizeof(TcTri),
+                                  cudaMemcpyHostToDevice, st));
+    TK_CUDA_CHECK(cudaMemcpyAsync(ws + L.range, pl.range.data(), pl.range.size() * sizeof(int),
+                                  cudaMemcpyHostToDevice, st));
+    const WsHeader h = plan_key(m, n, -2, -2, P);
+    TK_CUDA_CHECK(cudaMemcpyAsync(ws + offsetof(WsHeader, plan_m),
+                                  reinterpret_cast<const unsigned char *>(&h) + offsetof(WsHeader, plan_m),
+                                  offsetof(WsHeader, pad) - offsetof(WsHeader, plan_m), cudaMemcpyHostToDevice, st));
+    TK_CUDA_CHECK(cudaStreamSynchronize(st));  // the host plan lives in a cache that may be rebuilt
+    g_tcup[{dev, work}] = key;
+  }
+  // the other kernels' plan regions overlap this one
+  forget_plan(work);
+  forget_hessian_plan(work);
+  return TK_OK;
+}
+
 int contract_batched_tc(const BatchedArgs &a, cudaStream_t st) {
   DevInfo di;
   int rc = dev_info(&di);
@@ -649,35 +690,8 @@ int contract_batched_tc(const BatchedArgs &a, cudaStream_t st) {
   const TcLayout L = tc_layout(n, a.B, di.sms, njobs, ntris);
   if (a.work_bytes < L.total) return fail(TK_ENOMEM, "workspace %zu < %zu bytes (tensor-core batched pass)",
                                           a.work_bytes, L.total);
-  bool uploaded = false;
-  {
-  std::lock_guard<std::mutex> lk(g_tcmu);
-  TcKey key{m, n, P};
-  auto up = g_tcup.find({dev, a.work});
-  if (up == g_tcup.end() || up->second < key || key < up->second) {
-    const TcPlan &pl = tc_plan_for(m, n, P);
-    if (pl.jobs.size() != njobs || pl.tris.size() != ntris)
-      return fail(TK_EINVAL, "tensor-core plan: %zu jobs / %zu triangles, layout sized for %zu / %zu",
-                  pl.jobs.size(), pl.tris.size(), njobs, ntris);
-    TK_CUDA_CHECK(cudaMemcpyAsync(ws + L.jobs, pl.jobs.data(), pl.jobs.size() * sizeof(TcJob),
-                                  cudaMemcpyHostToDevice, st));
-    TK_CUDA_CHECK(cudaMemcpyAsync(ws + L.tris, pl.tris.data(), pl.tris.size() * sizeof(TcTri),
-                                  cudaMemcpyHostToDevice, st));
-    TK_CUDA_CHECK(cudaMemcpyAsync(ws + L.range, pl.range.data(), pl.range.size() * sizeof(int),
-                                  cudaMemcpyHostToDevice, st));
-    const WsHeader h = plan_key(m, n, -2, -2, P);
-    TK_CUDA_CHECK(cudaMemcpyAsync(ws + offsetof(WsHeader, plan_m),
-                                  reinterpret_cast<const unsigned char *>(&h) + offsetof(WsHeader, plan_m),
-                                  offsetof(WsHeader, pad) - offsetof(WsHeader, plan_m), cudaMemcpyHostToDevice, st));
-    TK_CUDA_CHECK(cudaStreamSynchronize(st));  // the host plan lives in a cache that may be rebuilt
-    g_tcup[{dev, a.work}] = key;
-    uploaded = true;
-  }
-  }
-  if (uploaded) {  // the other kernels' plan regions overlap this one
-    forget_plan(a.work);
-    forget_hessian_plan(a.work);
-  }
+  rc = tc_upload_plan(m, n, P, njobs, ntris, L, a.work, st);
+  if (rc != TK_OK) return rc;
   TcParams p;
   p.m = m;
   p.n = n;
@@ -713,7 +727,141 @@ int contract_batched_tc(const BatchedArgs &a, cudaStream_t st) {
   }
   TK_CUDA_CHECK(cudaGetLastError());
   dim3 rg((unsigned)((n + 1 + 127) / 128), (unsigned)a.B);
-  tc_reduce<<<rg, 128, 0, st>>>(m, n, n16, a.B, P, p.gpart, p.spart, a.vec_dtype, a.G, a.S, p.status);
+  tc_reduce<<<rg, 128, 0, st>>>(m, n, n16, a.B, kTcSlice, 1.0, P, p.gpart, p.spart, a.vec_dtype, a.G, a.S, p.status);
+  TK_CUDA_CHECK(cudaGetLastError());
+  return TK_OK;
+}
+
+// ------------------------------------------------------------------ FP32 rows pass
+// columns of a block, problems of a slice, slices and blocks per slice
+struct RgShape {
+  int NC, NP, slices, P;
+};
+static RgShape rg_shape(bool dual, int64_t B, int sms) {
+  RgShape r;
+  r.NC = B <= (dual ? 32 : 64) ? 64 : 128;
+  r.NP = dual ? r.NC / 2 : r.NC;
+  r.slices = (int)((B + r.NP - 1) / r.NP);
+  r.P = std::max(1, sms / r.slices);
+  return r;
+}
+
+struct RgLayout {
+  TcLayout t;
+  size_t g32, total;
+};
+static RgLayout rg_layout(int n, const RgShape &sh, size_t njobs, size_t ntris) {
+  auto al = [](size_t x) { return (x + 1023) & ~size_t(1023); };
+  const int n16 = (n + 15) & ~15, grid = sh.slices * sh.P;
+  RgLayout L;
+  size_t off = al(sizeof(WsHeader));
+  L.t.jobs = off;
+  off = al(off + njobs * sizeof(TcJob));
+  L.t.tris = off;
+  off = al(off + ntris * sizeof(TcTri));
+  L.t.range = off;
+  off = al(off + (size_t)(sh.P + 1) * sizeof(int));
+  L.t.img = off;
+  L.t.at = off;
+  off = al(off + (size_t)n * sh.slices * sh.NC * sizeof(float));
+  L.t.gpart = off;
+  off = al(off + (size_t)grid * n16 * kTcSlice * sizeof(double));
+  L.t.spart = off;
+  off = al(off + (size_t)grid * kTcSlice * sizeof(double));
+  L.g32 = off;
+  off = al(off + (size_t)grid * n16 * sh.NP * sizeof(float));
+  L.t.total = L.total = off;
+  return L;
+}
+
+// m = 3 and 4 from kRgMinN points: at higher orders most triangles fill little of a
+// job's 96 x 32 tiles.  Against the column-split kernel of tk_batched.cu (m = 4
+// FP32, B = 64, Hessian-vector product): n = 64 0.31 -> 0.14 ms, n = 100 0.83 ->
+// 0.38, n = 150 2.47 -> 1.02, n = 300 20.2 -> 10.0; contraction at B = 48 n = 100
+// 0.54 -> 0.39, n = 300 11.4 -> 8.8.
+bool rows_covers(int m, int n, int storage, bool dual, int64_t B, int64_t off_lo, int64_t off_hi) {
+  if (g_batched_cfg.tensor_cores < 0 || storage == TK_F64) return false;
+  if (off_lo != 0 || off_hi != multiset(n, m)) return false;  // whole tensor only
+  (void)dual;
+  return m >= 3 && m <= 4 && n >= kRgMinN && n <= kTcMaxN && B >= 1;
+}
+
+// The pass costs the same for 1 to 32 vectors (64 of the contraction); single
+// passes reach that at some n/16 (n/12) of them.  Measured, the pass against one
+// single pass (m = 4 FP32, Hessian-vector / contraction): n = 64 118 / 148 us
+// against 29 / 29, n = 100 0.28 / 0.39 ms against 0.041 / 0.042, n = 150 0.73 / 0.95
+// against 0.079 / 0.071, n = 300 6.9 / 8.8 against 0.49 / 0.36.
+bool rows_pays(int m, int n, int storage, bool dual, int64_t B, int64_t off_lo, int64_t off_hi) {
+  return g_batched_cfg.min_batch == 0 && rows_covers(m, n, storage, dual, B, off_lo, off_hi) &&
+         B * (dual ? 16 : 12) >= n;
+}
+
+size_t rows_workspace_bytes(int m, int n, int64_t B, int sms) {
+  size_t nj = 0, nt = 0;
+  tc_counts(m, n, &nj, &nt);
+  return std::max(rg_layout(n, rg_shape(false, B, sms), nj, nt).total,
+                  rg_layout(n, rg_shape(true, B, sms), nj, nt).total);
+}
+
+template <typename ST, bool DUAL, int NC>
+static int launch_rows(const RgParams &p, int grid, cudaStream_t st) {
+  const size_t smem = rg_smem<NC>(p.t.nkc);
+  TK_CUDA_CHECK(cudaFuncSetAttribute(rows_batched_kernel<ST, DUAL, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)smem));
+  rows_batched_kernel<ST, DUAL, NC><<<grid, kRgThreads, smem, st>>>(p);
+  TK_CUDA_CHECK(cudaGetLastError());
+  return TK_OK;
+}
+
+int contract_batched_rows(const BatchedArgs &a, cudaStream_t st) {
+  DevInfo di;
+  int rc = dev_info(&di);
+  if (rc != TK_OK) return rc;
+  const int m = a.m, n = a.n;
+  const bool dual = a.V != nullptr;
+  const RgShape sh = rg_shape(dual, a.B, di.sms);
+  size_t njobs = 0, ntris = 0;
+  tc_counts(m, n, &njobs, &ntris);
+  const RgLayout L = rg_layout(n, sh, njobs, ntris);
+  const int nkc = (n + 31) / 32, n16 = (n + 15) & ~15, Bpad = sh.slices * sh.NC, grid = sh.slices * sh.P;
+  if (a.work_bytes < L.total || rg_smem<128>(nkc) > (size_t)di.smem_optin)
+    return fail(TK_EUNSUPPORTED, "batched rows pass: workspace or shared memory");
+  unsigned char *ws = reinterpret_cast<unsigned char *>(a.work);
+  rc = tc_upload_plan(m, n, sh.P, njobs, ntris, L.t, a.work, st);
+  if (rc != TK_OK) return rc;
+  RgParams p;
+  p.t.m = m;
+  p.t.n = n;
+  p.t.n16 = n16;
+  p.t.nkc = nkc;
+  p.t.K = reinterpret_cast<const unsigned char *>(a.K);
+  p.t.jobs = reinterpret_cast<const TcJob *>(ws + L.t.jobs);
+  p.t.tris = reinterpret_cast<const TcTri *>(ws + L.t.tris);
+  p.t.range = reinterpret_cast<const int *>(ws + L.t.range);
+  p.t.P = sh.P;
+  p.t.slices = sh.slices;
+  p.t.Bpad = Bpad;
+  p.t.img = nullptr;
+  p.t.at = reinterpret_cast<const float *>(ws + L.t.at);
+  p.t.gpart = reinterpret_cast<double *>(ws + L.t.gpart);
+  p.t.spart = reinterpret_cast<double *>(ws + L.t.spart);
+  p.t.status = reinterpret_cast<int *>(ws);
+  p.g32 = reinterpret_cast<float *>(ws + L.g32);
+  rows_prep_vectors<<<(unsigned)(((int64_t)Bpad * n + 255) / 256), 256, 0, st>>>(
+      n, a.B, Bpad, sh.NC, sh.NP, a.vec_dtype, a.A, a.V, reinterpret_cast<float *>(ws + L.t.at));
+  TK_CUDA_CHECK(cudaGetLastError());
+  const bool f32 = a.storage == TK_F32;
+  if (dual) {
+    if (sh.NC == 128) rc = f32 ? launch_rows<float, true, 128>(p, grid, st) : launch_rows<__nv_bfloat16, true, 128>(p, grid, st);
+    else rc = f32 ? launch_rows<float, true, 64>(p, grid, st) : launch_rows<__nv_bfloat16, true, 64>(p, grid, st);
+  } else {
+    if (sh.NC == 128) rc = f32 ? launch_rows<float, false, 128>(p, grid, st) : launch_rows<__nv_bfloat16, false, 128>(p, grid, st);
+    else rc = f32 ? launch_rows<float, false, 64>(p, grid, st) : launch_rows<__nv_bfloat16, false, 64>(p, grid, st);
+  }
+  if (rc != TK_OK) return rc;
+  const dim3 rg((unsigned)((n + 1 + 127) / 128), (unsigned)a.B);
+  tc_reduce<<<rg, 128, 0, st>>>(m, n, n16, a.B, sh.NP, dual ? 1.0 / (m - 1) : 1.0, sh.P, p.t.gpart, p.t.spart,
+                                a.vec_dtype, a.G, dual ? nullptr : a.S, p.t.status);
   TK_CUDA_CHECK(cudaGetLastError());
   return TK_OK;
 }

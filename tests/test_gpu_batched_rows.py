@@ -1,0 +1,69 @@
+"""The FP32 rows pass (gathered rows of each triangle times all vectors): the
+contraction below the tensor cores' batch sizes and the Hessian-vector product, at
+the edges of its jobs, chunks and column halves."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+from gpu_util import U32, as_f64, round_storage
+
+pytestmark = pytest.mark.gpu
+
+tk = pytest.importorskip("paper_2003_10482_gb300")
+
+
+def rows_bound(abs_terms, n, m, dual):
+    """gamma_k times 2 sum |terms|.  k: a row dot of at most n + 31 products; in FP32
+    at most 64 jobs' additions into g and as many prefix terms between flushes, two
+    products each in the dual pass; the quadratic form's rows (6 per job and thread,
+    then 16 threads, at most n in all); the products of a term, 3m + 20, and the
+    product rule's 2m.  The 2: the quadratic form's absolute counterpart counts the
+    pairs of column b twice (once in the row sum, once in the a_b r_b correction)."""
+    k = (n + 31) + 4 * 64 + (n + 16) + 3 * m + 20 + (2 * m if dual else 0)
+    return 2 * 1.01 * k * U32 * abs_terms + 1e-30
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+@pytest.mark.parametrize("m,n,B,dual,vdt", [
+    (4, 40, 17, True, torch.float64), (4, 97, 32, True, torch.float32), (4, 65, 33, True, torch.float64),
+    (3, 128, 64, True, torch.float64), (3, 193, 70, True, torch.float64), (4, 64, 130, True, torch.float64),
+    (4, 63, 28, False, torch.float64), (4, 96, 63, False, torch.float32), (3, 129, 40, False, torch.float64),
+    (4, 41, 100, False, torch.float64)])
+def test_rows_pass_matches_oracle(m, n, B, dual, vdt, storage):
+    X = synth.small_problem(m, n, 3, salt=1100 + n)
+    Kt = round_storage(oracle.build(X, m), storage)
+    Kr = as_f64(Kt)
+    A = torch.tensor(synth.alpha_like(n, salt=1101, batch=B), device="cuda").to(vdt)
+    V = torch.tensor(synth.alpha_like(n, salt=1102, batch=B), device="cuda").to(vdt)
+    G, S = tk.tk_contract(Kt.cuda(), m, n, A, r=m - 2 if dual else None, V=V if dual else None)
+    assert tk.tk_status_read(tk.workspace(m, n, B)) == tk.TK_OK
+    G = G.double().cpu().numpy()
+    Ah, Vh = A.double().cpu().numpy(), V.double().cpu().numpy()
+    for b in sorted({0, 1, min(31, B - 1), B // 2, B - 1}):
+        if dual:
+            ref, mag = oracle.hvp(Kr, Ah[b], Vh[b], m), oracle.hvp(np.abs(Kr), np.abs(Ah[b]), np.abs(Vh[b]), m)
+        else:
+            ref, S_ref = oracle.contract(Kr, Ah[b], m)
+            mag, S_abs = oracle.contract(np.abs(Kr), np.abs(Ah[b]), m)
+            assert abs(float(S[b]) - S_ref) <= rows_bound(S_abs, n, m, dual)
+        tol = rows_bound(mag, n, m, dual) + (U32 * np.abs(ref) if vdt == torch.float32 else 0.0)
+        assert np.all(np.abs(G[b] - ref) <= tol), (b, float(np.max(np.abs(G[b] - ref) / tol)))
+
+
+def test_passes_share_one_workspace():
+    # single, rows, tensor-core and Hessian-vector passes in one workspace, in turn
+    m, n, B = 4, 70, 80
+    K = tk.tk_build_packed(torch.tensor(synth.small_problem(m, n, 3, salt=1110), device="cuda"), m, storage="f32")
+    A = torch.tensor(synth.alpha_like(n, salt=1111, batch=B), device="cuda")
+    work = tk.new_workspace(int(tk.lib().tk_contract_workspace_size(m, n, B)), A.device)
+    one = tk.tk_contract(K, m, n, A[:1], work=work)[0]
+    for b in (80, 40, 80, 16):
+        G, _ = tk.tk_contract(K, m, n, A[:b], work=work)
+        HV, _ = tk.tk_contract(K, m, n, A[:b], r=m - 2, V=A[:b], work=work)
+        again = tk.tk_contract(K, m, n, A[:1], work=work)[0]
+        assert torch.equal(again, one)
+        # Euler's identity: K[a^2, a] = K[a^3]
+        scale = float(G.abs().max())
+        assert torch.allclose(HV, G, rtol=0, atol=1e-4 * scale) and torch.allclose(G[:1], one, rtol=0, atol=1e-4 * scale)
