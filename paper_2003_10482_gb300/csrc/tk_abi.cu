@@ -138,7 +138,20 @@ size_t tk_contract_workspace_size(int m, int64_t n, int64_t B) {
   if (tc_covers(m, (int)n, TK_F32, false, B, 0, multiset(n, m))) need = std::max(need, tc_workspace_bytes(m, (int)n, B, di.sms));
   if (B > 1 && rows_covers(m, (int)n, TK_F32, false, B, 0, multiset(n, m)))
     need = std::max(need, rows_workspace_bytes(m, (int)n, B, di.sms));
+  const int64_t N = multiset(n, m);
+  if (pairs_covers(m, (int)n, TK_F32, 0, N)) need = std::max(need, pairs_workspace_bytes((int)n));
   return need;
+}
+
+// One vector's pass.
+static int single_pass(const ContractArgs &a, size_t work_bytes, cudaStream_t st) {
+  if (pairs_covers(a.m, a.n, a.storage, a.off_lo, a.off_hi)) {
+    const int rc = contract_pairs(a, work_bytes, st);
+    if (rc != TK_EUNSUPPORTED) return rc;
+  }
+  int grid = 0;
+  const double *part = nullptr;
+  return contract_pass(a, &grid, &part, st);
 }
 
 static int contract_impl(int m, int64_t n, int storage, const void *K, int64_t off_lo, int64_t off_hi,
@@ -220,9 +233,7 @@ static int contract_impl(int m, int64_t n, int storage, const void *K, int64_t o
     a.fin.out_dtype = vec_dtype;
     a.fin.G = reinterpret_cast<unsigned char *>(G) + b * n * vs;
     a.fin.S = (S && r == m - 1) ? S + b : nullptr;
-    int grid = 0;
-    const double *part = nullptr;
-    rc = contract_pass(a, &grid, &part, st);
+    rc = single_pass(a, work_bytes, st);
     if (rc != TK_OK) return rc;
   }
   return TK_OK;
@@ -375,9 +386,7 @@ int tk_objective(int m, int64_t n, int storage, const void *K, int64_t B, const 
     a.fin.F = F ? F + b : nullptr;
     a.fin.grad = grad ? grad + b * n : nullptr;
     a.fin.gnorm = gnorm ? gnorm + b : nullptr;
-    int grid = 0;
-    const double *part = nullptr;
-    rc = contract_pass(a, &grid, &part, st);
+    rc = single_pass(a, work_bytes, st);
     if (rc != TK_OK) return rc;
   }
   return TK_OK;

@@ -1,0 +1,434 @@
+// Contraction K[a^3], K[a^4] and Hessian-vector product K[a^2, v] at order m = 4
+// from the packed tensor as a matrix of prefixes x pairs (FP32 / BF16 storage,
+// whole tensor, larger n); tk_contract_impl.cuh serves the rest.
+//
+// The entries of a prefix Q = (i, b) are contiguous and run over the pairs
+// p = (c, d), b <= c <= d, in lexicographic order, the same for every i <= b.  With
+// the multiplicities of S(a) = sum_t mu(t) K_t a^t, mu = M'_Q f: f = 1 for c > b,
+// d > c; 1/2 for c = d > b; 1/(kb+1) for c = b < d; 1/((kb+1)(kb+2)) for c = d = b
+// (kb = cnt_Q(b), M' = 24, or 12 for i = b), two sums over that matrix hold it all:
+//   Y_b[p] = sum_i (M'/4) A_Q f K[Q][p]       (column sums, A_Q = a_i a_b)
+//   tau_Q  = sum_p f a_c a_d K[Q][p]          (row sums)
+// and with the symmetric matrices y = sum_b Y_b and tau
+//   g_l = sum_j y(l, j) a_j + 6 sum_j tau(l, j) a_j,   S = 12 a^T tau a
+// (the first sum over both orders of (l, j), y(l, l) twice).  Replacing a by
+// a + eps v and keeping the eps-coefficient gives the Hessian-vector product: Y'
+// and tau' beside Y and tau, from the same loads.
+//
+// So an entry costs a shared-memory load and two multiply-adds (four for the
+// product), with no triangles and no per-row work inside the loop: a warp holds one
+// tile of 512 pairs of one b -- Y and z_p = f a_c a_d in registers, 16 of each a
+// lane -- and walks the prefixes i = 0..b, one bulk copy of 2 KB (1 KB for BF16)
+// each into a ring of 10 KB.  Eight prefixes' row sums are reduced over the
+// lanes together (9 shuffles).  Every Y_b[p] and every (Q, tile) row sum belongs to
+// one warp: plain stores, no atomics, sums in a fixed order.  Two small kernels add
+// up Y over b, tau over the tiles (FP64) and form g, S and the objective.
+//
+// What bounds it: the contraction of FP32 storage HBM (the main kernel reads
+// 7.2 TB/s at n = 400, issue 45 % busy); the product and BF16 storage the per-prefix
+// work, some 3 to 4.4 prefix tiles per ns over the chip (110 to 170 instructions
+// each, 16 warps an SM held by Y, z and the ring).  Measured, streaming pass ->
+// this one: FP32 contraction n = 400 885 -> 685 us (objective call 874 -> 677),
+// n = 300 399 -> 264, n = 250 238 -> 177, n = 200 162 -> 141; Hessian-vector product
+// n = 400 1037 -> 775, n = 351 701 -> 499, n = 250 276 -> 237, n = 200 188 -> 192 (below,
+// the four launches cost more than they save); BF16 n = 600 2852 -> 2424, its product
+// 3616 -> 3547, n = 400 741 -> 548 and 958 -> 788.  Loads into registers instead of
+// the ring (1 KB or 2 KB a prefix, one to four in flight) read 4.4 to 4.7 TB/s; the
+// same walk over b for a fixed i 3.7.
+#include <cuda_bf16.h>
+#include <stddef.h>
+
+#include <algorithm>
+
+#include "tk_prefix.cuh"
+
+namespace tk {
+
+constexpr int kPT = 512;        // pairs per tile
+constexpr int kPC = kPT / 32;   // of them a lane's
+// prefixes in flight a warp: 10 KB, 160 an SM
+template <typename ST>
+constexpr int kPNB = sizeof(ST) == 4 ? 5 : 10;
+constexpr int kPRow = 8;        // prefixes whose row sums are reduced together
+constexpr int kPMinN = 200;     // points from which the pass is taken (see the figures above)
+constexpr int kPMaxN = 640;     // and to which (its sums take up to 5 % of the tensor's bytes)
+
+struct PParams {
+  int n;
+  int64_t pairs;
+  const unsigned char *K;
+  const void *alpha, *v;
+  int vec_dtype;
+  int64_t *slab;         // [n] slab of i as if its triangles began at b = 0
+  float *z, *zd;         // [pairs] f a_c a_d of c > b, and its derivative
+  float *Y, *Yd;         // [item][kPT]
+  float *t, *td;         // [item][n] the tile's part of tau(i, b), at i
+  double *y, *yd;        // [pairs]
+  double *tau, *taud;    // [pairs] (i, b), i <= b: index b (b + 1) / 2 + i
+  double *part;          // [3][n + 2] g (or the product) and S
+  WsHeader *hdr;
+  FinalizeArgs fin;
+  int64_t bytes;         // of K
+  int item[kPMaxN + 1];  // items (tiles) of the values above b (item[n]: all)
+};
+
+// z of every pair, the slabs, and the workspace's plan key voided
+template <bool D>
+__global__ void __launch_bounds__(256) pairs_prep(PParams p) {
+  const int n = p.n;
+  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < n) {
+    const int64_t i = q;
+    p.slab[i] = multiset(n, 4) - multiset(n - i, 4) - (multiset(n, 3) - multiset(n - i, 3));
+  }
+  if (q == 0) {
+    p.hdr->plan_m = 0;
+    p.hdr->done = 0;
+  }
+  if (q >= p.pairs) return;
+  const int c = pair_row(n, (int)q), d = c + (int)q - pair_start(n, c);
+  const float f = c == d ? 0.5f : 1.f;
+  const float ac = ld_vec<float>(p.alpha, p.vec_dtype, c), ad = ld_vec<float>(p.alpha, p.vec_dtype, d);
+  p.z[q] = f * ac * ad;
+  if (D) p.zd[q] = f * (ac * ld_vec<float>(p.v, p.vec_dtype, d) + ld_vec<float>(p.v, p.vec_dtype, c) * ad);
+}
+
+template <typename ST, bool D>
+__global__ void __launch_bounds__(256, 2) pairs_kernel(PParams p) {
+  constexpr int NB = kPNB<ST>;
+  using Ring = RowRing<ST, kPT, NB>;
+  extern __shared__ __align__(16) unsigned char pk_smem[];
+  const int n = p.n, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int64_t *slab = reinterpret_cast<int64_t *>(pk_smem + 8 * Ring::kWarpBytes);
+  float *a_s = reinterpret_cast<float *>(slab + n), *v_s = a_s + n;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    a_s[i] = ld_vec<float>(p.alpha, p.vec_dtype, i);
+    if (D) v_s[i] = ld_vec<float>(p.v, p.vec_dtype, i);
+    slab[i] = p.slab[i];
+  }
+  Ring ring;
+  ring.init(pk_smem + w * Ring::kWarpBytes, p.K, p.bytes, lane);
+  __syncthreads();
+  const int item = blockIdx.x * 8 + w;
+  if (item >= p.item[n]) return;
+  // b descending (the longest walks first): the smallest b with item >= item[b]
+  int b;
+  {
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (p.item[mid] <= item) hi = mid; else lo = mid + 1;
+    }
+    b = lo;
+  }
+  const int t = item - p.item[b];
+  const int L = n - b, np = L * (L + 1) / 2;
+  const int p0 = t * kPT + lane, count = min(kPT, np - t * kPT);
+  const ST *K = reinterpret_cast<const ST *>(p.K) + (int)(multiset(n, 3) - multiset(L, 3)) + t * kPT;
+
+  float z[kPC], zd[kPC], Y[kPC], Yd[kPC];
+  {
+    const float *zp = p.z + pair_start(n, b) + p0, *zdp = p.zd + pair_start(n, b) + p0;
+#pragma unroll
+    for (int k = 0; k < kPC; ++k) {
+      const int q = p0 + 32 * k;
+      const float f = q == 0 ? 1.f / 3.f : q < L ? 0.5f : 1.f;  // the row c = b at kb = 1
+      z[k] = q < np ? f * zp[32 * k] : 0.f;
+      zd[k] = D && q < np ? f * zdp[32 * k] : 0.f;
+      Y[k] = Yd[k] = 0.f;
+    }
+  }
+  const float ab = 6.f * a_s[b], vb = D ? 6.f * v_s[b] : 0.f;
+  float *tp = p.t + (size_t)item * n, *tdp = p.td + (size_t)item * n;
+  for (int i = 0; i < min(NB, b + 1); ++i) ring.issue(i, K + slab[i], count);
+  int slot = 0;
+  uint32_t phase = 0;
+  bool ok = true;
+  for (int i0 = 0; i0 <= b && ok; i0 += kPRow) {
+    float s[kPRow], sd[kPRow];
+#pragma unroll
+    for (int r = 0; r < kPRow; ++r) {
+      s[r] = sd[r] = 0.f;
+      const int i = i0 + r;
+      if (i <= b && ok) {
+        const ST *xp = ring.take(slot, phase, K + slab[i], &ok) + lane;
+        float x[kPC];
+        if (count == kPT) {
+#pragma unroll
+          for (int k = 0; k < kPC; ++k) x[k] = ld_elem<ST, float>(xp + 32 * k);
+        } else {
+#pragma unroll
+          for (int k = 0; k < kPC; ++k) x[k] = lane + 32 * k < count ? ld_elem<ST, float>(xp + 32 * k) : 0.f;
+        }
+        if (i + NB <= b) ring.issue(slot, K + slab[i + NB], count);
+        if (++slot == NB) {
+          slot = 0;
+          phase ^= 1u;
+        }
+        float ca = ab * a_s[i], cd = D ? vb * a_s[i] + ab * v_s[i] : 0.f;
+        if (i == b) {
+          // Q = (b, b): M' is half, and the row c = b has kb = 2 (f = 1/3, 1/12)
+          ca *= 0.5f;
+          cd *= 0.5f;
+#pragma unroll
+          for (int k = 0; k < kPC; ++k) {
+            const int q = p0 + 32 * k;
+            if (q < L) x[k] *= q == 0 ? 0.5f : 2.f / 3.f;
+          }
+        }
+        float s0 = 0.f, s1 = 0.f, d0 = 0.f, d1 = 0.f;
+#pragma unroll
+        for (int k = 0; k < kPC; ++k) {
+          Y[k] = __fmaf_rn(ca, x[k], Y[k]);
+          if (k & 1) s1 = __fmaf_rn(z[k], x[k], s1); else s0 = __fmaf_rn(z[k], x[k], s0);
+          if (D) {
+            Yd[k] = __fmaf_rn(cd, x[k], Yd[k]);
+            if (k & 1) d1 = __fmaf_rn(zd[k], x[k], d1); else d0 = __fmaf_rn(zd[k], x[k], d0);
+          }
+        }
+        s[r] = s0 + s1;
+        if (D) sd[r] = d0 + d1;
+      }
+    }
+    const float v = warp_scatter8(s, lane);
+    const int i = i0 + (lane >> 2);
+    if ((lane & 3) == 0 && i <= b) tp[i] = v;
+    if (D) {
+      const float vd = warp_scatter8(sd, lane);
+      if ((lane & 3) == 0 && i <= b) tdp[i] = vd;
+    }
+  }
+  if (!ok) {
+    if (lane == 0) {
+      atomicExch(&p.hdr->status, TK_ETIMEOUT);
+      p.hdr->where = kSiteContractWait;
+    }
+    ring.drain(slot, phase);
+  }
+  // the row weights at kb = 1 (c = d is weighted with y)
+  float *yp = p.Y + (size_t)item * kPT + lane, *ydp = p.Yd + (size_t)item * kPT + lane;
+#pragma unroll
+  for (int k = 0; k < kPC; ++k) {
+    const int q = p0 + 32 * k;
+    const float f = q == 0 ? 1.f / 3.f : q < L ? 0.5f : 1.f;
+    yp[32 * k] = f * Y[k];
+    if (D) ydp[32 * k] = f * Yd[k];
+  }
+}
+
+// y of every pair (sums over b <= c) and tau of every prefix (sums over its
+// tiles): 32 of them a block, 8 warps over the summands in FP32 runs of 8, FP64
+// beyond.  Blocks [0, half) take pairs, the others prefixes.
+template <bool D>
+__global__ void __launch_bounds__(256) pairs_sum(PParams p, int half) {
+  __shared__ double sm[2][8][33];
+  const int n = p.n, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const bool is_y = (int)blockIdx.x < half;
+  const int g = 32 * (is_y ? blockIdx.x : blockIdx.x - half) + lane;
+  int cnt = 0, c = 0, i = 0;
+  if (g < p.pairs) {
+    if (is_y) {
+      c = pair_row(n, g);
+      cnt = c + 1;
+    } else {
+      c = (int)((sqrtf(8.f * (float)g + 1.f) - 1.f) * 0.5f);
+      while (c * (c + 1) / 2 > g) --c;
+      while ((c + 1) * (c + 2) / 2 <= g) ++c;
+      i = g - c * (c + 1) / 2;
+      cnt = pair_tiles(n, c, kPT);
+    }
+  }
+  // summand j: Y of b = j, or tile j of the prefix (i, c)
+  auto at = [&](int j) -> size_t {
+    return is_y ? (size_t)p.item[j] * kPT + (g - pair_start(n, j)) : (size_t)(p.item[c] + j) * n + i;
+  };
+  const float *src = is_y ? p.Y : p.t, *srd = is_y ? p.Yd : p.td;
+  double y = 0.0, yd = 0.0;
+  for (int j0 = w; j0 < cnt; j0 += 64) {
+    float v[8], vd[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int j = j0 + 8 * k;
+      const size_t o = at(min(j, cnt - 1));
+      v[k] = src[o];
+      vd[k] = D ? srd[o] : 0.f;
+    }
+    float s = 0.f, sd = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (j0 + 8 * k < cnt) {
+        s += v[k];
+        sd += vd[k];
+      }
+    }
+    y += (double)s;
+    if (D) yd += (double)sd;
+  }
+  sm[0][w][lane] = y;
+  if (D) sm[1][w][lane] = yd;
+  __syncthreads();
+  if (w < (D ? 2 : 1) && g < p.pairs) {
+    double t = 0.0;
+    for (int k = 0; k < 8; ++k) t += sm[w][k][lane];
+    if (is_y) (w ? p.yd : p.y)[g] = (g == pair_start(n, c) ? 0.5 : 1.0) * t;
+    else (w ? p.taud : p.tau)[g] = t;
+  }
+}
+
+// g_l (or the product's entry l) and a_l's share of S, one block per l; the last
+// block writes the outputs
+template <bool D>
+__global__ void __launch_bounds__(128) pairs_final(PParams p) {
+  const int n = p.n, l = blockIdx.x;
+  auto av = [&](int j) { return ld_vec<double>(p.alpha, p.vec_dtype, j); };
+  auto vv = [&](int j) { return ld_vec<double>(p.v, p.vec_dtype, j); };
+  double g = 0.0, ts = 0.0;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    const int lo = min(l, j), hi = max(l, j);
+    const int64_t q = pair_start(n, lo) + hi - lo, h = (int64_t)hi * (hi + 1) / 2 + lo;
+    const double two = l == j ? 2.0 : 1.0;
+    // (tau(l, l) stands for both orders of its one prefix already)
+    if (D) {
+      g += two * (p.y[q] * vv(j) + p.yd[q] * av(j)) + 6.0 * (p.tau[h] * vv(j) + p.taud[h] * av(j));
+    } else {
+      const double ta = p.tau[h] * av(j);
+      g += two * p.y[q] * av(j) + 6.0 * ta;
+      ts += ta;
+    }
+  }
+  __shared__ double sg[4], st[4];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    g += __shfl_xor_sync(0xffffffffu, g, o);
+    ts += __shfl_xor_sync(0xffffffffu, ts, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    sg[threadIdx.x >> 5] = g;
+    st[threadIdx.x >> 5] = ts;
+  }
+  __syncthreads();
+  __shared__ int s_last;
+  if (threadIdx.x == 0) {
+    // partials laid out as the blocks' of the streaming pass: [vec][n + 2] of one
+    // "block", S as a_l-weighted shares
+    p.part[(D ? n + 2 : 0) + l] = sg[0] + sg[1] + sg[2] + sg[3];
+    p.part[2 * (n + 2) + l] = D ? 0.0 : 12.0 * av(l) * (st[0] + st[1] + st[2] + st[3]);
+    __threadfence();
+    s_last = atomicAdd(&p.hdr->done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (threadIdx.x < 32) {
+    double S = 0.0;
+    for (int j = threadIdx.x; j < n; j += 32) S += __ldcg(p.part + 2 * (n + 2) + j);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) S += __shfl_xor_sync(0xffffffffu, S, o);
+    if (threadIdx.x == 0) p.part[n] = S;
+    __threadfence();
+  }
+  __syncthreads();
+  final_reduce(p.fin, p.part, 1);
+}
+
+// ------------------------------------------------------------------ host
+struct PLayout {
+  size_t slab, z, zd, Y, Yd, t, td, y, yd, tau, taud, part, total;
+};
+
+static PLayout pairs_layout(int n, bool dual) {
+  auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
+  const size_t pairs = (size_t)n * (n + 1) / 2;
+  size_t items = 0;
+  for (int i = 0; i < n; ++i) items += pair_tiles(n, i, kPT);
+  PLayout P;
+  size_t off = sizeof(WsHeader);
+  auto take = [&](size_t bytes) {
+    const size_t at = off;
+    off = al(off + bytes);
+    return at;
+  };
+  P.slab = take((size_t)n * 8);
+  P.y = take(pairs * 8);
+  P.tau = take(pairs * 8);
+  P.part = take((size_t)3 * (n + 2) * 8);
+  P.z = take(pairs * 4);
+  P.Y = take(items * kPT * 4);
+  P.t = take(items * n * 4);
+  P.yd = take(dual ? pairs * 8 : 0);
+  P.taud = take(dual ? pairs * 8 : 0);
+  P.zd = take(dual ? pairs * 4 : 0);
+  P.Yd = take(dual ? items * kPT * 4 : 0);
+  P.td = take(dual ? items * n * 4 : 0);
+  P.total = off;
+  return P;
+}
+
+bool pairs_covers(int m, int n, int storage, int64_t off_lo, int64_t off_hi) {
+  return m == 4 && storage != TK_F64 && n >= kPMinN && n <= kPMaxN && off_lo == 0 && off_hi == multiset(n, m);
+}
+
+size_t pairs_workspace_bytes(int n) { return pairs_layout(n, true).total; }
+
+template <typename ST, bool D>
+static int launch_pairs(const PParams &p, cudaStream_t st) {
+  pairs_prep<D><<<(unsigned)((p.pairs + 255) / 256), 256, 0, st>>>(p);
+  TK_CUDA_CHECK(cudaGetLastError());
+  const size_t smem = 8 * RowRing<ST, kPT, kPNB<ST>>::kWarpBytes + p.n * (sizeof(int64_t) + (D ? 2 : 1) * sizeof(float));
+  TK_CUDA_CHECK(cudaFuncSetAttribute(pairs_kernel<ST, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  pairs_kernel<ST, D><<<(unsigned)((p.item[p.n] + 7) / 8), 256, smem, st>>>(p);
+  TK_CUDA_CHECK(cudaGetLastError());
+  const int half = (int)((p.pairs + 31) / 32);
+  pairs_sum<D><<<(unsigned)(2 * half), 256, 0, st>>>(p, half);
+  TK_CUDA_CHECK(cudaGetLastError());
+  pairs_final<D><<<(unsigned)p.n, 128, 0, st>>>(p);
+  TK_CUDA_CHECK(cudaGetLastError());
+  return TK_OK;
+}
+
+int contract_pairs(const ContractArgs &a, size_t work_bytes, cudaStream_t st) {
+  const bool dual = a.v != nullptr;
+  const PLayout L = pairs_layout(a.n, dual);
+  if (L.total > work_bytes) return fail(TK_EUNSUPPORTED, "pairs pass: workspace");
+  // the pass overwrites any plan of this workspace (its first launch voids the key)
+  forget_plan(a.work);
+  forget_tc_plan(a.work);
+  forget_hessian_plan(a.work);
+  unsigned char *ws = reinterpret_cast<unsigned char *>(a.work);
+  PParams p;
+  p.n = a.n;
+  p.pairs = (int64_t)a.n * (a.n + 1) / 2;
+  p.bytes = a.off_hi * dtype_size(a.storage);
+  int items = 0;
+  for (int b = a.n - 1; b >= 0; --b) {
+    p.item[b] = items;
+    items += pair_tiles(a.n, b, kPT);
+  }
+  p.item[a.n] = items;
+  p.K = reinterpret_cast<const unsigned char *>(a.K);
+  p.alpha = a.alpha;
+  p.v = a.v;
+  p.vec_dtype = a.vec_dtype;
+  p.slab = reinterpret_cast<int64_t *>(ws + L.slab);
+  p.z = reinterpret_cast<float *>(ws + L.z);
+  p.zd = reinterpret_cast<float *>(ws + L.zd);
+  p.Y = reinterpret_cast<float *>(ws + L.Y);
+  p.Yd = reinterpret_cast<float *>(ws + L.Yd);
+  p.t = reinterpret_cast<float *>(ws + L.t);
+  p.td = reinterpret_cast<float *>(ws + L.td);
+  p.y = reinterpret_cast<double *>(ws + L.y);
+  p.yd = reinterpret_cast<double *>(ws + L.yd);
+  p.tau = reinterpret_cast<double *>(ws + L.tau);
+  p.taud = reinterpret_cast<double *>(ws + L.taud);
+  p.part = reinterpret_cast<double *>(ws + L.part);
+  p.hdr = reinterpret_cast<WsHeader *>(ws);
+  p.fin = a.fin;
+  p.fin.part = p.part;
+  p.fin.grid = 1;
+  p.fin.m = a.m;
+  p.fin.n = a.n;
+  if (a.storage == TK_F32) return dual ? launch_pairs<float, true>(p, st) : launch_pairs<float, false>(p, st);
+  return dual ? launch_pairs<__nv_bfloat16, true>(p, st) : launch_pairs<__nv_bfloat16, false>(p, st);
+}
+
+}  // namespace tk

@@ -165,6 +165,13 @@ struct ContractArgs {
 // part[block][vec][n + 2]: vec 0 = value, vec 1 = derivative; entry n = S).
 int contract_pass(const ContractArgs &a, int *grid_out, const double **part_out, cudaStream_t st);
 
+// The same pass (FP32/BF16 storage, whole tensor, larger sizes) over the tensor as
+// a matrix of prefixes x pairs (order 4); TK_EUNSUPPORTED when the workspace is too
+// small for it.
+bool pairs_covers(int m, int n, int storage, int64_t off_lo, int64_t off_hi);
+size_t pairs_workspace_bytes(int n);
+int contract_pairs(const ContractArgs &a, size_t work_bytes, cudaStream_t st);
+
 // Process-wide overrides of the contraction launch configuration.
 extern tk_contract_config g_contract_cfg;
 // Resolve the configuration of a pass (no launch); fills the kernel's ring,

@@ -1,0 +1,104 @@
+// Shared by the single-vector passes over the tensor as a matrix of prefixes x
+// pairs (tk_contract_pairs.cu, tk_contract_prefix.cu): the pairs' order, a warp's
+// ring of row segments in shared memory and its row-sum reduction.
+#pragma once
+#include "tk_contract_impl.cuh"
+
+namespace tk {
+
+// index of the pair (b, b) among the pairs (c, d), c <= d, in lexicographic order
+TK_HD int pair_start(int n, int b) { return (int)((int64_t)b * (2 * n - b + 1) / 2); }
+
+// first value of the pair with index q: the largest c with pair_start(c) <= q
+TK_HD int pair_row(int n, int q) {
+  int c = 0, hi = n - 1;
+  while (c < hi) {
+    const int mid = (c + hi + 1) >> 1;
+    if (pair_start(n, mid) <= q) c = mid; else hi = mid - 1;
+  }
+  return c;
+}
+
+// tiles of T pairs of the triangles with last prefix value b
+TK_HD int pair_tiles(int n, int b, int T) { return ((n - b) * (n - b + 1) / 2 + T - 1) / T; }
+
+// A warp's ring of NB row segments of at most T entries, each fetched by one
+// cp.async.bulk of the 16-byte-aligned bytes around it.
+template <typename ST, int T, int NB>
+struct RowRing {
+  static constexpr int kBytes = T * (int)sizeof(ST) + 32;
+  static constexpr int kWarpBytes = NB * kBytes + ((NB * 8 + 15) & ~15);
+  unsigned char *buf;
+  uint64_t *bar;
+  const unsigned char *tail;  // the array's last 16-byte boundary
+  int lane;
+
+  __device__ void init(unsigned char *warp_smem, const void *K, int64_t bytes, int lane_) {
+    buf = warp_smem;
+    bar = reinterpret_cast<uint64_t *>(warp_smem + NB * kBytes);
+    tail = reinterpret_cast<const unsigned char *>(K) + (bytes & ~int64_t(15));
+    lane = lane_;
+    if (lane == 0) {
+      for (int s = 0; s < NB; ++s) mbar_init(&bar[s], 1);
+      fence_barrier_init();
+    }
+    __syncwarp();
+  }
+  // start the copy of `count` entries at src into slot s (every lane has read the
+  // slot's last segment and calls)
+  __device__ __forceinline__ void issue(int s, const ST *src, int count) {
+    const unsigned char *p = reinterpret_cast<const unsigned char *>(src);
+    const uint32_t lead = (uint32_t)reinterpret_cast<uintptr_t>(p) & 15u;
+    uint32_t bytes = (lead + (uint32_t)count * (uint32_t)sizeof(ST) + 15u) & ~15u;
+    unsigned char *dst = buf + s * kBytes;
+    __syncwarp();
+    if (p - lead + bytes > tail) bytes = by_hand(dst, p - lead, p + (size_t)count * sizeof(ST));
+    if (lane == 0) {
+      fence_proxy_async();
+      if (bytes) {
+        mbar_expect_tx(&bar[s], bytes);
+        bulk_g2s(dst, p - lead, bytes, &bar[s]);
+      } else {
+        mbar_arrive(&bar[s]);
+      }
+    }
+  }
+  // the segment [b0, e) reaches past the boundary (the array's last one): its bytes
+  // from there on are copied by hand; returns the bulk copy's
+  __device__ __noinline__ uint32_t by_hand(unsigned char *dst, const unsigned char *b0, const unsigned char *e) {
+    const uint32_t bytes = b0 < tail ? (uint32_t)(tail - b0) : 0u;
+    if (lane < (int)(e - (b0 + bytes))) dst[bytes + lane] = b0[bytes + lane];
+    __syncwarp();
+    return bytes;
+  }
+  // the segment in slot s, once its copy of the given phase has landed
+  __device__ __forceinline__ const ST *take(int s, uint32_t phase, const ST *src, bool *ok) {
+    *ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[s], phase));
+    return reinterpret_cast<const ST *>(buf + s * kBytes + ((uint32_t)reinterpret_cast<uintptr_t>(src) & 15u));
+  }
+  // after a wait that ran out: give the copies in flight from slot s on their
+  // time before the block can end
+  __device__ __noinline__ void drain(int s, uint32_t phase) {
+    for (int k = 0; k < NB; ++k)
+      mbar_wait_bounded(&bar[(s + k) % NB], phase ^ (s + k >= NB ? 1u : 0u));
+  }
+};
+
+// Sum of the 8 values of every lane over the warp: lane l ends with value l >> 2's
+__device__ __forceinline__ float warp_scatter8(float (&v)[8], int lane) {
+#pragma unroll
+  for (int k = 16, cnt = 4; cnt >= 1; k >>= 1, cnt >>= 1) {
+    const bool up = (lane & k) != 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (j < cnt) {
+        const float send = up ? v[j] : v[j + cnt], keep = up ? v[j + cnt] : v[j];
+        v[j] = keep + __shfl_xor_sync(0xffffffffu, send, k);
+      }
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+}  // namespace tk
