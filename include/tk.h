@@ -190,8 +190,9 @@ int tk_contract_range(int m, int64_t n, int storage_dtype, const void *K_range,
                       void *work, size_t work_bytes, void *stream);
 
 /* Launch configuration of the streaming contraction kernel (single vectors;
- * not of the pass that takes whole FP32 / BF16 tensors of order 4, 200 <= n <=
- * 640, in its place).  Zero fields keep the library's choice.
+ * not of the passes that take FP32 / BF16 tensors of order 4, 200 <= n <= 640,
+ * and whole tensors of 5e7 entries of orders from 5 on in its place).  Zero
+ * fields keep the library's choice.
  *   warps        warps per block (each warp walks its own row-aligned piece)
  *   block_bytes  bytes of one staging buffer (one bulk copy per row block), a
  *                multiple of 128 in [1024, 65536]; 0 = the largest that fits

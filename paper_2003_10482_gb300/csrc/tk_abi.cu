@@ -140,6 +140,7 @@ size_t tk_contract_workspace_size(int m, int64_t n, int64_t B) {
     need = std::max(need, rows_workspace_bytes(m, (int)n, B, di.sms));
   const int64_t N = multiset(n, m);
   if (pairs_covers(m, (int)n, TK_F32, 0, N)) need = std::max(need, pairs_workspace_bytes((int)n));
+  if (prefix_covers(m, (int)n, TK_F32, false, 0, N)) need = std::max(need, prefix_workspace_bytes(m, (int)n, di.sms));
   return need;
 }
 
@@ -147,6 +148,10 @@ size_t tk_contract_workspace_size(int m, int64_t n, int64_t B) {
 static int single_pass(const ContractArgs &a, size_t work_bytes, cudaStream_t st) {
   if (pairs_covers(a.m, a.n, a.storage, a.off_lo, a.off_hi)) {
     const int rc = contract_pairs(a, work_bytes, st);
+    if (rc != TK_EUNSUPPORTED) return rc;
+  }
+  if (prefix_covers(a.m, a.n, a.storage, a.v != nullptr, a.off_lo, a.off_hi)) {
+    const int rc = contract_prefix(a, work_bytes, st);
     if (rc != TK_EUNSUPPORTED) return rc;
   }
   int grid = 0;

@@ -1,0 +1,484 @@
+// Contraction K[a^{m-1}], K[a^m] at orders m >= 5 by prefixes and pairs (FP32 /
+// BF16 storage, whole tensor); tk_contract_impl.cuh serves the rest.
+//
+// At high orders the tensor is many small triangles (m = 6, n = 80: 1.8 million of
+// some 240 entries), and the streaming pass spends its time on their rows.  But the
+// entries of a prefix Q = (q_1..q_{m-3}, b) are contiguous and run over the pairs
+// p = (c, d), b <= c <= d, in lexicographic order, the same pairs for every prefix
+// of one b.  With mu(t) = M'_Q f the multiplicity of a stored tuple (M'_Q =
+// m!/prod_v cnt_Q(v)!; f = 1 for c > b, d > c; 1/2 for c = d > b; 1/(kb+1) for
+// c = b < d; 1/((kb+1)(kb+2)) for c = d = b, kb = cnt_Q(b)) two sums hold all of it:
+//   Y_b[p] = sum_Q (M'_Q/m) A_Q f K[Q][p]    (prefixes with last value b)
+//   tau_Q  = sum_p f a_c a_d K[Q][p]
+// The c and d positions give g_l = sum_j y(l, j) a_j, y = sum_b Y_b (both orders,
+// y(l, l) twice); the prefix positions are those of the order-(m-2) tensor tau:
+// M'_Q = m (m-1) mu_{m-2}(Q), so they add (m-1)(m-2) tau[a^{m-3}], and
+// S = m (m-1) tau[a^{m-2}], which a pass of the streaming kernel over tau computes.
+//
+// A warp holds a tile of 256 pairs of one b (Y and z_p = f a_c a_d of kb = 1, 8 of
+// each a lane) and walks a run of prefixes, one load and two multiply-adds per
+// entry, one bulk copy per prefix into a ring of six.  A prefix's offset is a sum of m - 3 table
+// values,  base(Q) = C(n+m-1, m) - sum_j W_j[q_j] - C(n-b+2, 3),
+// W_j[x] = C(n-1-x + m-j-1, m-j), its index in tau likewise; 32 lanes form the
+// next 32 prefixes' offsets and coefficients together.  Plain stores, fixed order.
+//
+// What bounds it: the work per (prefix, tile) -- its copy's issue and wait, the
+// broadcasts of its record -- at some 150 entries each.  Measured, streaming pass ->
+// this one: m = 6, n = 80 1970 -> 1266 us (1.75 GB), n = 60 584 -> 461, BF16 n = 80
+// 2026 -> 1277; m = 5, n = 100 333 -> 290.  At m = 6, n = 45 the six launches took 254
+// against 201 us: hence kXMinEntries.
+#include <cuda_bf16.h>
+#include <stddef.h>
+
+#include <algorithm>
+
+#include "tk_prefix.cuh"
+
+namespace tk {
+
+constexpr int kXC = 8;              // chunks of 32 pairs per tile
+constexpr int kXT = 32 * kXC;
+constexpr int kXNB = 6;             // prefixes in flight a warp
+constexpr int kXSlices = 32;        // slices of b in the sums of y
+constexpr int kXMaxN = 256;
+constexpr int64_t kXMinEntries = 50000000;  // entries from which the pass is taken
+
+struct XParams {
+  int m, n;
+  int64_t size;         // entries
+  int64_t pairs, nq;    // pairs of n points, prefixes (entries of tau)
+  const unsigned char *K;
+  const void *alpha;
+  int vec_dtype;
+  float *z;             // [pairs] f a_c a_d of c > b
+  float *Y;             // [item][kXT]
+  float *t;             // [tile][nq] the tile's part of tau
+  float *tau;           // [nq], 16-byte aligned
+  double *y;            // [kXSlices][pairs]
+  double *g2;           // [n] tau[a^{m-3}], then [n] its S
+  double *part;         // [3][n + 2]
+  WsHeader *hdr;
+  unsigned int *done;   // blocks of the last launch that have finished
+  FinalizeArgs fin;
+  int rows;             // prefixes (about) per item
+  int item[kXMaxN + 1]; // items of the values below b
+};
+
+// (m-4)-prefixes per item of b, and items per tile
+TK_HD int64_t x_leads(int m, int b) { return multiset(b + 1, m - 4); }
+TK_HD int x_step(int b, int rows) { return rows / (b + 1) + 1; }
+TK_HD int x_splits(int m, int b, int rows) { return (int)((x_leads(m, b) + x_step(b, rows) - 1) / x_step(b, rows)); }
+
+__global__ void __launch_bounds__(256) prefix_prep(XParams p) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q == 0) *p.done = 0;
+  if (q >= p.pairs) return;
+  const int c = pair_row(p.n, q), d = c + q - pair_start(p.n, c);
+  p.z[q] = (c == d ? 0.5f : 1.f) * ld_vec<float>(p.alpha, p.vec_dtype, c) * ld_vec<float>(p.alpha, p.vec_dtype, d);
+}
+
+template <typename ST>
+__global__ void __launch_bounds__(256, 3) prefix_kernel(XParams p) {
+  __shared__ float a_s[kXMaxN];
+  __shared__ int64_t W[kMaxOrder - 3][kXMaxN];  // offset of a prefix value at position j
+  __shared__ int V[kMaxOrder - 3][kXMaxN];      // its part of the index in tau
+  const int n = p.n, m = p.m, lane = threadIdx.x & 31;
+  for (int e = threadIdx.x; e < n; e += blockDim.x) a_s[e] = ld_vec<float>(p.alpha, p.vec_dtype, e);
+  for (int e = threadIdx.x; e < (m - 3) * n; e += blockDim.x) {
+    const int j = e / n, x = e - j * n;
+    W[j][x] = multiset(n - 1 - x, m - j);
+    V[j][x] = (int)multiset(n - 1 - x, m - 2 - j);
+  }
+  __syncthreads();
+  extern __shared__ __align__(16) unsigned char xk_smem[];
+  RowRing<ST, kXT, kXNB> ring;
+  ring.init(xk_smem + (threadIdx.x >> 5) * RowRing<ST, kXT, kXNB>::kWarpBytes, p.K, p.size * (int64_t)sizeof(ST), lane);
+  const int item = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (item >= p.item[n]) return;
+  int b;
+  {
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (p.item[mid] <= item) lo = mid; else hi = mid - 1;
+    }
+    b = lo;
+  }
+  const int nt = pair_tiles(n, b, kXT);
+  const int sp = (item - p.item[b]) / nt, t = item - p.item[b] - sp * nt;
+  const int L = n - b, np = L * (L + 1) / 2, p0 = t * kXT + lane;
+  const bool first_row = t * kXT < L;
+  float z[kXC], Y[kXC];
+#pragma unroll
+  for (int k = 0; k < kXC; ++k) {
+    const int q = p0 + 32 * k;
+    z[k] = q < np ? p.z[pair_start(n, b) + q] * (q == 0 ? 1.f / 3.f : q < L ? 0.5f : 1.f) : 0.f;
+    Y[k] = 0.f;
+  }
+  const ST *K = reinterpret_cast<const ST *>(p.K) + (p.size - multiset(n - b, 3)) + t * kXT;
+  float *tp = p.t + (size_t)t * p.nq + (p.nq - (n - b));
+  float mfact = 1.f;  // m! / m
+  for (int j = 2; j < m; ++j) mfact *= (float)j;
+  const float ab = a_s[b];
+
+  // the (m-4)-prefixes [l0, l1) of the item; within one, the values u..b of the
+  // last free position
+  const int64_t leads = x_leads(m, b), l0 = (int64_t)sp * x_step(b, p.rows);
+  const int64_t l1 = min(leads, l0 + x_step(b, p.rows));
+  int32_t ld[kMaxOrder];
+  unrank(m - 4, b + 1, l0, ld);
+  int u = ld[m - 5];
+  int64_t l = l0;
+  bool more = true;
+  // lane j: the record of the j-th prefix of a batch of 32: offset, index,
+  // coefficient, multiplicity of b (the current batch and the next)
+  struct Rec {
+    int64_t off;
+    int idx, kb, cnt;
+    float coef;
+  } cur, nxt;
+  // fill up to 32 records: runs of consecutive last values, several leads if they fit
+  auto fill = [&](Rec &rec) {
+    int cnt = 0;
+    rec.off = 0;
+    rec.idx = 0;
+    rec.kb = 1;
+    rec.coef = 0.f;
+    while (cnt < 32 && more) {
+      const int take = min(32 - cnt, b - u + 1);
+      if (lane >= cnt && lane < cnt + take) {
+        const int x = u + lane - cnt;
+        int64_t o = W[m - 4][x];
+        int id = V[m - 4][x];
+        float A = 1.f, den = 1.f;
+        int run = 0, kbx = 1, prev = -1;
+        for (int j = 0; j < m - 4; ++j) {
+          o += W[j][ld[j]];
+          id += V[j][ld[j]];
+          A *= a_s[ld[j]];
+          run = ld[j] == prev ? run + 1 : 1;
+          den *= (float)run;
+          kbx += ld[j] == b;
+          prev = ld[j];
+        }
+        A *= a_s[x];
+        run = x == prev ? run + 1 : 1;
+        den *= (float)run;
+        kbx += x == b;
+        if (x == b) den *= (float)(run + 1);
+        rec.off = -o;
+        rec.idx = -id;
+        rec.kb = kbx;
+        rec.coef = A * ab * (mfact / den);
+      }
+      cnt += take;
+      u += take;
+      if (u > b) {
+        if (++l < l1) {
+          next_sorted(m - 4, b + 1, ld);
+          u = ld[m - 5];
+        } else {
+          more = false;
+        }
+      }
+    }
+    rec.cnt = cnt;
+  };
+  const int count = min(kXT, np - t * kXT);
+  int slot = 0;  // of the next segment
+  uint32_t phase = 0;
+  bool ok = true;
+  fill(cur);
+  fill(nxt);
+  // (a batch that another one follows is full, and longer than the ring)
+  for (int i = 0; i < min(kXNB, cur.cnt); ++i) ring.issue(i, K + __shfl_sync(0xffffffffu, cur.off, i), count);
+  while (cur.cnt > 0 && ok) {
+    const int cnt = cur.cnt;
+    const uint32_t multi = __ballot_sync(0xffffffffu, lane < cnt && cur.kb > 1);
+    for (int r0 = 0; r0 < cnt; r0 += 8) {
+      float s[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const int i = r0 + r;
+        s[r] = 0.f;
+        if (i < cnt && ok) {
+          const ST *xp = ring.take(slot, phase, K + __shfl_sync(0xffffffffu, cur.off, i), &ok) + lane;
+          float x[kXC];
+          if (count == kXT) {
+#pragma unroll
+            for (int k = 0; k < kXC; ++k) x[k] = ld_elem<ST, float>(xp + 32 * k);
+          } else {
+#pragma unroll
+            for (int k = 0; k < kXC; ++k) x[k] = lane + 32 * k < count ? ld_elem<ST, float>(xp + 32 * k) : 0.f;
+          }
+          // the slot takes the prefix kXNB further on, of this batch or the next
+          const int f = i + kXNB - cnt;
+          if (f < nxt.cnt) ring.issue(slot, K + __shfl_sync(0xffffffffu, f < 0 ? cur.off : nxt.off, f < 0 ? f + cnt : f), count);
+          if (++slot == kXNB) {
+            slot = 0;
+            phase ^= 1u;
+          }
+          const float ca = __shfl_sync(0xffffffffu, cur.coef, i);
+          if (first_row && (multi >> i & 1)) {
+            const float k1 = (float)__shfl_sync(0xffffffffu, cur.kb, i);
+            const float w1 = 2.f / (k1 + 1.f), w0 = 6.f / ((k1 + 1.f) * (k1 + 2.f));
+#pragma unroll
+            for (int k = 0; k < kXC; ++k) {
+              const int q = p0 + 32 * k;
+              if (q < L) x[k] *= q == 0 ? w0 : w1;
+            }
+          }
+          float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+          for (int k = 0; k < kXC; ++k) {
+            Y[k] = __fmaf_rn(ca, x[k], Y[k]);
+            if (k & 1) s1 = __fmaf_rn(z[k], x[k], s1); else s0 = __fmaf_rn(z[k], x[k], s0);
+          }
+          s[r] = s0 + s1;
+        }
+      }
+      const float v = warp_scatter8(s, lane);
+      const int j = r0 + (lane >> 2), at = __shfl_sync(0xffffffffu, cur.idx, j & 31);
+      if ((lane & 3) == 0 && j < cnt) tp[at] = v;
+    }
+    cur = nxt;
+    fill(nxt);
+  }
+  if (!ok) {
+    if (lane == 0) {
+      atomicExch(&p.hdr->status, TK_ETIMEOUT);
+      p.hdr->where = kSiteContractWait;
+    }
+    ring.drain(slot, phase);
+  }
+  float *yp = p.Y + (size_t)item * kXT + lane;
+#pragma unroll
+  for (int k = 0; k < kXC; ++k) {
+    const int q = p0 + 32 * k;
+    yp[32 * k] = (q == 0 ? 1.f / 3.f : q < L ? 0.5f : 1.f) * Y[k];
+  }
+}
+
+// tau of every prefix: its tiles' parts.  A warp takes kXRun consecutive values of
+// the packed order, in which the last value b runs fastest.
+constexpr int kXRun = 256;
+__global__ void __launch_bounds__(256) prefix_tau(XParams p) {
+  const int lane = threadIdx.x & 31;
+  int64_t h0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * kXRun;
+  const int64_t h1 = min(h0 + kXRun, p.nq);
+  if (h0 >= h1) return;
+  int32_t q[kMaxOrder];
+  unrank(p.m - 2, p.n, h0, q);
+  int b0 = q[p.m - 3];
+  for (; h0 < h1; h0 += 32) {
+    int b = 0;
+    for (int have = 0; have < 32;) {
+      const int take = min(32 - have, p.n - b0);
+      if (lane >= have && lane < have + take) b = b0 + lane - have;
+      have += take;
+      b0 += take;
+      if (b0 == p.n) {
+        if (!next_sorted(p.m - 3, p.n, q)) break;
+        b0 = q[p.m - 4];
+      }
+    }
+    const int64_t h = h0 + lane;
+    if (h >= h1) continue;
+    const int nt = pair_tiles(p.n, b, kXT);
+    double s = 0.0;
+    for (int t0 = 0; t0 < nt; t0 += 8) {
+      float v[8], u = 0.f;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = t0 + j < nt ? p.t[(size_t)(t0 + j) * p.nq + h] : 0.f;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) u += v[j];
+      s += (double)u;
+    }
+    p.tau[h] = (float)s;
+  }
+}
+
+// y of every pair: sums over b <= c and their items, a slice of the b per block
+// (32 pairs, 8 warps over the items)
+__global__ void __launch_bounds__(256) prefix_y(XParams p) {
+  __shared__ double sm[8][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int g = blockIdx.x * 32 + lane;
+  double y = 0.0;
+  if (g < p.pairs) {
+    const int c = pair_row(p.n, g);
+    for (int b = blockIdx.y; b <= c; b += kXSlices) {
+      const int q = g - pair_start(p.n, b), nt = pair_tiles(p.n, b, kXT), ns = x_splits(p.m, b, p.rows);
+      const float *src = p.Y + (size_t)(p.item[b] + q / kXT) * kXT + q % kXT;
+      for (int s0 = w; s0 < ns; s0 += 64) {
+        float v[8], s = 0.f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = src[(size_t)min(s0 + 8 * j, ns - 1) * nt * kXT];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (s0 + 8 * j < ns) s += v[j];
+        y += (double)s;
+      }
+    }
+  }
+  sm[w][lane] = y;
+  __syncthreads();
+  if (w == 0 && g < p.pairs) {
+    double t = 0.0;
+    for (int j = 0; j < 8; ++j) t += sm[j][lane];
+    p.y[(size_t)blockIdx.y * p.pairs + g] = t;
+  }
+}
+
+// g_l, one block per l; the last block writes the outputs
+__global__ void __launch_bounds__(128) prefix_final(XParams p) {
+  const int n = p.n, l = blockIdx.x;
+  double g = 0.0;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    const int lo = min(l, j), hi = max(l, j);
+    // (y(l, l) twice, weighted 1/2)
+    double y = 0.0;
+    for (int s = 0; s < kXSlices; ++s) y += p.y[(size_t)s * p.pairs + pair_start(n, lo) + hi - lo];
+    g += y * ld_vec<double>(p.alpha, p.vec_dtype, j);
+  }
+  __shared__ double sg[4];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+  if ((threadIdx.x & 31) == 0) sg[threadIdx.x >> 5] = g;
+  __syncthreads();
+  __shared__ int s_last;
+  if (threadIdx.x == 0) {
+    p.part[l] = sg[0] + sg[1] + sg[2] + sg[3] + (double)((p.m - 1) * (p.m - 2)) * p.g2[l];
+    if (l == 0) p.part[n] = (double)(p.m * (p.m - 1)) * p.g2[n];
+    __threadfence();
+    s_last = atomicAdd(p.done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  final_reduce(p.fin, p.part, 1);
+}
+
+// ------------------------------------------------------------------ host
+struct XLayout {
+  size_t done, z, Y, t, tau, y, g2, part, total;
+};
+
+// prefixes per item: some four items for each of the 24 warps per SM
+static int prefix_rows(int m, int n, int sms) {
+  int64_t total = 0;
+  for (int b = 0; b < n; ++b) total += multiset(b + 1, m - 3) * pair_tiles(n, b, kXT);
+  return (int)std::max<int64_t>(32, std::min<int64_t>(1024, total / ((int64_t)sms * 48)));
+}
+
+static XLayout prefix_layout(int m, int n, int sms) {
+  auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
+  const size_t pairs = (size_t)n * (n + 1) / 2, nq = (size_t)multiset(n, m - 2);
+  const int rows = prefix_rows(m, n, sms);
+  size_t items = 0;
+  for (int b = 0; b < n; ++b) items += (size_t)pair_tiles(n, b, kXT) * x_splits(m, b, rows);
+  XLayout X;
+  // the front is the workspace of the streaming pass over tau
+  size_t off = al(contract_workspace_bytes(n, sms));
+  auto take = [&](size_t bytes) {
+    const size_t at = off;
+    off = al(off + bytes);
+    return at;
+  };
+  X.done = take(sizeof(unsigned int));
+  X.z = take(pairs * 4);
+  X.y = take(kXSlices * pairs * 8);
+  X.g2 = take((size_t)(n + 1) * 8);
+  X.part = take((size_t)3 * (n + 2) * 8);
+  X.Y = take(items * kXT * 4);
+  X.t = take((size_t)pair_tiles(n, 0, kXT) * nq * 4);
+  X.tau = take(nq * 4);
+  X.total = off;
+  return X;
+}
+
+bool prefix_covers(int m, int n, int storage, bool dual, int64_t off_lo, int64_t off_hi) {
+  return m >= 5 && !dual && storage != TK_F64 && n <= kXMaxN && off_lo == 0 && off_hi == multiset(n, m) &&
+         off_hi >= kXMinEntries;
+}
+
+size_t prefix_workspace_bytes(int m, int n, int sms) { return prefix_layout(m, n, sms).total; }
+
+template <typename ST>
+static int launch_prefix(const XParams &p, unsigned grid, cudaStream_t st) {
+  constexpr int smem = 8 * RowRing<ST, kXT, kXNB>::kWarpBytes;
+  TK_CUDA_CHECK(cudaFuncSetAttribute(prefix_kernel<ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  prefix_kernel<ST><<<grid, 256, smem, st>>>(p);
+  TK_CUDA_CHECK(cudaGetLastError());
+  return TK_OK;
+}
+
+int contract_prefix(const ContractArgs &a, size_t work_bytes, cudaStream_t st) {
+  DevInfo di;
+  int rc = dev_info(&di);
+  if (rc != TK_OK) return rc;
+  const XLayout L = prefix_layout(a.m, a.n, di.sms);
+  if (L.total > work_bytes) return fail(TK_EUNSUPPORTED, "prefix pass: workspace");
+  // the arrays lie over those of the batched and Hessian passes
+  forget_tc_plan(a.work);
+  forget_hessian_plan(a.work);
+  unsigned char *ws = reinterpret_cast<unsigned char *>(a.work);
+  XParams p;
+  p.m = a.m;
+  p.n = a.n;
+  p.size = a.off_hi;
+  p.pairs = (int64_t)a.n * (a.n + 1) / 2;
+  p.nq = multiset(a.n, a.m - 2);
+  p.K = reinterpret_cast<const unsigned char *>(a.K);
+  p.alpha = a.alpha;
+  p.vec_dtype = a.vec_dtype;
+  p.z = reinterpret_cast<float *>(ws + L.z);
+  p.Y = reinterpret_cast<float *>(ws + L.Y);
+  p.t = reinterpret_cast<float *>(ws + L.t);
+  p.tau = reinterpret_cast<float *>(ws + L.tau);
+  p.y = reinterpret_cast<double *>(ws + L.y);
+  p.g2 = reinterpret_cast<double *>(ws + L.g2);
+  p.part = reinterpret_cast<double *>(ws + L.part);
+  p.hdr = reinterpret_cast<WsHeader *>(ws);
+  p.done = reinterpret_cast<unsigned int *>(ws + L.done);
+  p.fin = a.fin;
+  p.fin.part = p.part;
+  p.fin.grid = 1;
+  p.fin.m = a.m;
+  p.fin.n = a.n;
+  p.rows = prefix_rows(a.m, a.n, di.sms);
+  p.item[0] = 0;
+  for (int b = 0; b < a.n; ++b) p.item[b + 1] = p.item[b] + pair_tiles(a.n, b, kXT) * x_splits(a.m, b, p.rows);
+  const unsigned gp = (unsigned)((p.pairs + 255) / 256);
+  prefix_prep<<<gp, 256, 0, st>>>(p);
+  TK_CUDA_CHECK(cudaGetLastError());
+  const unsigned gk = (unsigned)((p.item[a.n] + 7) / 8);
+  if (a.storage == TK_F32) rc = launch_prefix<float>(p, gk, st);
+  else rc = launch_prefix<__nv_bfloat16>(p, gk, st);
+  if (rc != TK_OK) return rc;
+  TK_CUDA_CHECK(cudaGetLastError());
+  prefix_tau<<<(unsigned)((p.nq + 8 * kXRun - 1) / (8 * kXRun)), 256, 0, st>>>(p);
+  TK_CUDA_CHECK(cudaGetLastError());
+  prefix_y<<<dim3((unsigned)((p.pairs + 31) / 32), kXSlices), 256, 0, st>>>(p);
+  TK_CUDA_CHECK(cudaGetLastError());
+  // tau[a^{m-3}] and tau[a^{m-2}]
+  ContractArgs t = a;
+  t.m = a.m - 2;
+  t.storage = TK_F32;
+  t.K = p.tau;
+  t.off_lo = 0;
+  t.off_hi = p.nq;
+  t.v = nullptr;
+  t.fin = FinalizeArgs{};
+  t.fin.mode = 0;
+  t.fin.out_dtype = TK_F64;
+  t.fin.G = p.g2;
+  t.fin.S = p.g2 + a.n;
+  rc = contract_pass(t, nullptr, nullptr, st);
+  if (rc != TK_OK) return rc;
+  prefix_final<<<(unsigned)a.n, 128, 0, st>>>(p);
+  TK_CUDA_CHECK(cudaGetLastError());
+  return TK_OK;
+}
+
+}  // namespace tk

@@ -166,11 +166,14 @@ struct ContractArgs {
 int contract_pass(const ContractArgs &a, int *grid_out, const double **part_out, cudaStream_t st);
 
 // The same pass (FP32/BF16 storage, whole tensor, larger sizes) over the tensor as
-// a matrix of prefixes x pairs (order 4); TK_EUNSUPPORTED when the workspace is too
-// small for it.
+// a matrix of prefixes x pairs: order 4 with the Hessian-vector product, orders
+// from 5 on without; TK_EUNSUPPORTED when the workspace is too small for them.
 bool pairs_covers(int m, int n, int storage, int64_t off_lo, int64_t off_hi);
 size_t pairs_workspace_bytes(int n);
 int contract_pairs(const ContractArgs &a, size_t work_bytes, cudaStream_t st);
+bool prefix_covers(int m, int n, int storage, bool dual, int64_t off_lo, int64_t off_hi);
+size_t prefix_workspace_bytes(int m, int n, int sms);
+int contract_prefix(const ContractArgs &a, size_t work_bytes, cudaStream_t st);
 
 // Process-wide overrides of the contraction launch configuration.
 extern tk_contract_config g_contract_cfg;
