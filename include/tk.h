@@ -28,7 +28,7 @@
  *     stream).  Device calls are asynchronous on that stream unless noted.
  *   - Device buffers must be 16-byte aligned (every cudaMalloc / PyTorch
  *     allocation is).
- *   - No floating-point atomics; every reduction runs in a fixed order, and
+ *   - No floating-point atomics (but in tk_hessian); every reduction runs in a fixed order, and
  *     with the default schedule (tk_contract_config.schedule) results are
  *     bit-reproducible from run to run.
  */
@@ -400,9 +400,10 @@ int tk_dual_hvp(int m, int64_t n, int storage_dtype, const void *K, int64_t B, c
  * a dense symmetric n x n FP64 matrix (row-major, device), from one pass over
  * the packed tensor (each entry read once).  a: n FP64 (device).  Arithmetic
  * as in tk_contract (FP32 with FP64 cross-block sums for FP32/BF16 storage);
- * the few entries whose rows and columns are both prefix values
- * (i, j <= the triangle's last prefix value) are summed with FP64 atomic
- * adds, so they may vary in the last bits from run to run.  n up to 768
+ * all entries at orders 3 and 4, and at the others the few whose rows and
+ * columns are both prefix values (i, j <= the triangle's last prefix value),
+ * are summed with FP64 atomic adds, so they may vary in the last bits from run
+ * to run.  n up to 768
  * (FP32/BF16 storage) or 384 (FP64 storage), else TK_EUNSUPPORTED.
  * Workspace: tk_hessian_workspace_size bytes, which carry a cached work plan
  * like the contraction's. */

@@ -185,6 +185,32 @@ int plan_to_device(int m, int n, int64_t lo, int64_t hi, int pieces, int row_cos
   return ensure_plan(key, work, st);
 }
 
+__global__ void set_plan_key(WsHeader *hdr, int m, int n, long long tag) {
+  hdr->plan_m = m;
+  hdr->plan_n = n;
+  hdr->plan_pieces = 0;
+  hdr->plan_lo = hdr->plan_hi = tag;
+}
+
+int claim_workspace(int m, int n, int64_t tag, void *work, cudaStream_t st) {
+  const PlanKey key{m, n, tag, tag, 0, 0, 0};
+  int dev = 0;
+  TK_CUDA_CHECK(cudaGetDevice(&dev));
+  void *plan_region = reinterpret_cast<unsigned char *>(work) + sizeof(WsHeader);
+  {
+    std::lock_guard<std::mutex> lk(g_plan_mu);
+    auto up = g_uploaded.find({dev, plan_region});
+    if (up != g_uploaded.end() && up->second == key) return TK_OK;
+  }
+  forget_hessian_plan(work);
+  forget_tc_plan(work);
+  std::lock_guard<std::mutex> lk(g_plan_mu);
+  set_plan_key<<<1, 1, 0, st>>>(reinterpret_cast<WsHeader *>(work), m, n, tag);
+  TK_CUDA_CHECK(cudaGetLastError());
+  g_uploaded[{dev, plan_region}] = key;
+  return TK_OK;
+}
+
 void forget_plan(void *work) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return;
@@ -325,6 +351,14 @@ static int launch_pass(const ContractArgs &a, const KParams &kp, const Resolved 
   if (a.storage == TK_F64) return contract_launch_f64(kp, dual, r.nc, r.grid, r.warps * 32, r.smem, st);
   if (a.storage == TK_F32) return contract_launch_f32(kp, dual, r.nc, r.grid, r.warps * 32, r.smem, st);
   return contract_launch_bf16(kp, dual, r.nc, r.grid, r.warps * 32, r.smem, st);
+}
+
+int contract_plan(const ContractArgs &a, int *pieces, cudaStream_t st) {
+  Resolved r;
+  int rc = resolve(a.m, a.n, a.storage, a.v != nullptr, &r);
+  if (rc != TK_OK) return rc;
+  *pieces = r.ppw * r.grid * r.warps;
+  return ensure_plan(PlanKey{a.m, a.n, a.off_lo, a.off_hi, *pieces, r.row_cost, r.tri_cost}, a.work, st);
 }
 
 int contract_pass(const ContractArgs &a, int *grid_out, const double **part_out, cudaStream_t st) {

@@ -72,19 +72,22 @@ struct PParams {
   int item[kPMaxN + 1];  // items (tiles) of the values above b (item[n]: all)
 };
 
-// z of every pair, the slabs, and the workspace's plan key voided
+// whether the workspace has become another pass's (every kernel then returns)
+__device__ __forceinline__ bool pairs_stale(const PParams &p) {
+  return plan_is_stale(&p.hdr->status, 4, p.n, 0, kPairsTag, kPairsTag);
+}
+
+// z of every pair and the slabs
 template <bool D>
 __global__ void __launch_bounds__(256) pairs_prep(PParams p) {
+  if (pairs_stale(p)) return;
   const int n = p.n;
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (q < n) {
     const int64_t i = q;
     p.slab[i] = multiset(n, 4) - multiset(n - i, 4) - (multiset(n, 3) - multiset(n - i, 3));
   }
-  if (q == 0) {
-    p.hdr->plan_m = 0;
-    p.hdr->done = 0;
-  }
+  if (q == 0) p.hdr->done = 0;
   if (q >= p.pairs) return;
   const int c = pair_row(n, (int)q), d = c + (int)q - pair_start(n, c);
   const float f = c == d ? 0.5f : 1.f;
@@ -98,6 +101,7 @@ __global__ void __launch_bounds__(256, 2) pairs_kernel(PParams p) {
   constexpr int NB = kPNB<ST>;
   using Ring = RowRing<ST, kPT, NB>;
   extern __shared__ __align__(16) unsigned char pk_smem[];
+  if (pairs_stale(p)) return;
   const int n = p.n, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int64_t *slab = reinterpret_cast<int64_t *>(pk_smem + 8 * Ring::kWarpBytes);
   float *a_s = reinterpret_cast<float *>(slab + n), *v_s = a_s + n;
@@ -222,6 +226,7 @@ __global__ void __launch_bounds__(256, 2) pairs_kernel(PParams p) {
 template <bool D>
 __global__ void __launch_bounds__(256) pairs_sum(PParams p, int half) {
   __shared__ double sm[2][8][33];
+  if (pairs_stale(p)) return;
   const int n = p.n, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const bool is_y = (int)blockIdx.x < half;
   const int g = 32 * (is_y ? blockIdx.x : blockIdx.x - half) + lane;
@@ -279,6 +284,7 @@ __global__ void __launch_bounds__(256) pairs_sum(PParams p, int half) {
 // block writes the outputs
 template <bool D>
 __global__ void __launch_bounds__(128) pairs_final(PParams p) {
+  if (pairs_stale(p)) return;
   const int n = p.n, l = blockIdx.x;
   auto av = [&](int j) { return ld_vec<double>(p.alpha, p.vec_dtype, j); };
   auto vv = [&](int j) { return ld_vec<double>(p.v, p.vec_dtype, j); };
@@ -390,10 +396,8 @@ int contract_pairs(const ContractArgs &a, size_t work_bytes, cudaStream_t st) {
   const bool dual = a.v != nullptr;
   const PLayout L = pairs_layout(a.n, dual);
   if (L.total > work_bytes) return fail(TK_EUNSUPPORTED, "pairs pass: workspace");
-  // the pass overwrites any plan of this workspace (its first launch voids the key)
-  forget_plan(a.work);
-  forget_tc_plan(a.work);
-  forget_hessian_plan(a.work);
+  const int rc = claim_workspace(4, a.n, kPairsTag, a.work, st);
+  if (rc != TK_OK) return rc;
   unsigned char *ws = reinterpret_cast<unsigned char *>(a.work);
   PParams p;
   p.n = a.n;

@@ -61,6 +61,7 @@ struct XParams {
   unsigned int *done;   // blocks of the last launch that have finished
   FinalizeArgs fin;
   int rows;             // prefixes (about) per item
+  int pieces;           // of the streaming pass's plan over tau
   int item[kXMaxN + 1]; // items of the values below b
 };
 
@@ -69,7 +70,13 @@ TK_HD int64_t x_leads(int m, int b) { return multiset(b + 1, m - 4); }
 TK_HD int x_step(int b, int rows) { return rows / (b + 1) + 1; }
 TK_HD int x_splits(int m, int b, int rows) { return (int)((x_leads(m, b) + x_step(b, rows) - 1) / x_step(b, rows)); }
 
+// whether the workspace's plan has become another pass's (every kernel then returns)
+__device__ __forceinline__ bool prefix_stale(const XParams &p) {
+  return plan_is_stale(&p.hdr->status, p.m - 2, p.n, p.pieces, 0, p.nq);
+}
+
 __global__ void __launch_bounds__(256) prefix_prep(XParams p) {
+  if (prefix_stale(p)) return;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q == 0) *p.done = 0;
   if (q >= p.pairs) return;
@@ -82,6 +89,7 @@ __global__ void __launch_bounds__(256, 3) prefix_kernel(XParams p) {
   __shared__ float a_s[kXMaxN];
   __shared__ int64_t W[kMaxOrder - 3][kXMaxN];  // offset of a prefix value at position j
   __shared__ int V[kMaxOrder - 3][kXMaxN];      // its part of the index in tau
+  if (prefix_stale(p)) return;
   const int n = p.n, m = p.m, lane = threadIdx.x & 31;
   for (int e = threadIdx.x; e < n; e += blockDim.x) a_s[e] = ld_vec<float>(p.alpha, p.vec_dtype, e);
   for (int e = threadIdx.x; e < (m - 3) * n; e += blockDim.x) {
@@ -263,6 +271,7 @@ __global__ void __launch_bounds__(256, 3) prefix_kernel(XParams p) {
 // the packed order, in which the last value b runs fastest.
 constexpr int kXRun = 256;
 __global__ void __launch_bounds__(256) prefix_tau(XParams p) {
+  if (prefix_stale(p)) return;
   const int lane = threadIdx.x & 31;
   int64_t h0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * kXRun;
   const int64_t h1 = min(h0 + kXRun, p.nq);
@@ -301,6 +310,7 @@ __global__ void __launch_bounds__(256) prefix_tau(XParams p) {
 // y of every pair: sums over b <= c and their items, a slice of the b per block
 // (32 pairs, 8 warps over the items)
 __global__ void __launch_bounds__(256) prefix_y(XParams p) {
+  if (prefix_stale(p)) return;
   __shared__ double sm[8][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int g = blockIdx.x * 32 + lane;
@@ -332,6 +342,7 @@ __global__ void __launch_bounds__(256) prefix_y(XParams p) {
 
 // g_l, one block per l; the last block writes the outputs
 __global__ void __launch_bounds__(128) prefix_final(XParams p) {
+  if (prefix_stale(p)) return;
   const int n = p.n, l = blockIdx.x;
   double g = 0.0;
   for (int j = threadIdx.x; j < n; j += blockDim.x) {
@@ -419,9 +430,6 @@ int contract_prefix(const ContractArgs &a, size_t work_bytes, cudaStream_t st) {
   if (rc != TK_OK) return rc;
   const XLayout L = prefix_layout(a.m, a.n, di.sms);
   if (L.total > work_bytes) return fail(TK_EUNSUPPORTED, "prefix pass: workspace");
-  // the arrays lie over those of the batched and Hessian passes
-  forget_tc_plan(a.work);
-  forget_hessian_plan(a.work);
   unsigned char *ws = reinterpret_cast<unsigned char *>(a.work);
   XParams p;
   p.m = a.m;
@@ -449,19 +457,8 @@ int contract_prefix(const ContractArgs &a, size_t work_bytes, cudaStream_t st) {
   p.rows = prefix_rows(a.m, a.n, di.sms);
   p.item[0] = 0;
   for (int b = 0; b < a.n; ++b) p.item[b + 1] = p.item[b] + pair_tiles(a.n, b, kXT) * x_splits(a.m, b, p.rows);
-  const unsigned gp = (unsigned)((p.pairs + 255) / 256);
-  prefix_prep<<<gp, 256, 0, st>>>(p);
-  TK_CUDA_CHECK(cudaGetLastError());
-  const unsigned gk = (unsigned)((p.item[a.n] + 7) / 8);
-  if (a.storage == TK_F32) rc = launch_prefix<float>(p, gk, st);
-  else rc = launch_prefix<__nv_bfloat16>(p, gk, st);
-  if (rc != TK_OK) return rc;
-  TK_CUDA_CHECK(cudaGetLastError());
-  prefix_tau<<<(unsigned)((p.nq + 8 * kXRun - 1) / (8 * kXRun)), 256, 0, st>>>(p);
-  TK_CUDA_CHECK(cudaGetLastError());
-  prefix_y<<<dim3((unsigned)((p.pairs + 31) / 32), kXSlices), 256, 0, st>>>(p);
-  TK_CUDA_CHECK(cudaGetLastError());
-  // tau[a^{m-3}] and tau[a^{m-2}]
+  // tau[a^{m-3}] and tau[a^{m-2}]: the plan of that pass first, its key is this
+  // pass's too (the arrays lie over those of the batched and Hessian passes)
   ContractArgs t = a;
   t.m = a.m - 2;
   t.storage = TK_F32;
@@ -474,6 +471,20 @@ int contract_prefix(const ContractArgs &a, size_t work_bytes, cudaStream_t st) {
   t.fin.out_dtype = TK_F64;
   t.fin.G = p.g2;
   t.fin.S = p.g2 + a.n;
+  rc = contract_plan(t, &p.pieces, st);
+  if (rc != TK_OK) return rc;
+  const unsigned gp = (unsigned)((p.pairs + 255) / 256);
+  prefix_prep<<<gp, 256, 0, st>>>(p);
+  TK_CUDA_CHECK(cudaGetLastError());
+  const unsigned gk = (unsigned)((p.item[a.n] + 7) / 8);
+  if (a.storage == TK_F32) rc = launch_prefix<float>(p, gk, st);
+  else rc = launch_prefix<__nv_bfloat16>(p, gk, st);
+  if (rc != TK_OK) return rc;
+  TK_CUDA_CHECK(cudaGetLastError());
+  prefix_tau<<<(unsigned)((p.nq + 8 * kXRun - 1) / (8 * kXRun)), 256, 0, st>>>(p);
+  TK_CUDA_CHECK(cudaGetLastError());
+  prefix_y<<<dim3((unsigned)((p.pairs + 31) / 32), kXSlices), 256, 0, st>>>(p);
+  TK_CUDA_CHECK(cudaGetLastError());
   rc = contract_pass(t, nullptr, nullptr, st);
   if (rc != TK_OK) return rc;
   prefix_final<<<(unsigned)a.n, 128, 0, st>>>(p);

@@ -598,12 +598,7 @@ extern "C" int tk_hessian(int m, int64_t n, int storage, const void *K, const do
   if (takes_hessian34(m)) {
     const size_t need = sizeof(WsHeader) + (size_t)n * n * sizeof(double);
     if (work_bytes < need) return fail(TK_ENOMEM, "workspace %zu < %zu bytes", work_bytes, need);
-    // the sums overwrite any plan this workspace held: its key goes with it
-    forget_plan(work);
-    forget_tc_plan(work);
-    forget_hessian_plan(work);
-    TK_CUDA_CHECK(cudaMemsetAsync(ws + offsetof(WsHeader, plan_m), 0, need - offsetof(WsHeader, plan_m), st));
-    return hessian34(m, (int)n, storage, K, alpha, H, reinterpret_cast<double *>(ws + sizeof(WsHeader)), st);
+    return hessian34(m, (int)n, storage, K, alpha, H, work, st);
   }
   // the Hessian plan occupies the same region of a workspace as the
   // contraction plans: whatever those recorded for this address is void

@@ -55,6 +55,7 @@ struct H34Params {
   const unsigned char *K;
   const double *alpha;
   double *Z;
+  WsHeader *hdr;
   int pre[kH34MaxQ + 1];  // items before each row block
 };
 
@@ -89,6 +90,7 @@ template <typename ST, typename CT, int M, int NI, int MINB>
 __global__ void __launch_bounds__(256, MINB) hess34_kernel(H34Params p) {
   constexpr int NR = kH34Rows;
   extern __shared__ __align__(16) unsigned char h34_smem[];
+  if (plan_is_stale(&p.hdr->status, M, p.n, 0, kHessian34Tag, kHessian34Tag)) return;
   CT *a_s = reinterpret_cast<CT *>(h34_smem);
   const int n = p.n, lane = threadIdx.x & 31;
   for (int i = threadIdx.x; i < n; i += blockDim.x) a_s[i] = (CT)p.alpha[i];
@@ -279,8 +281,14 @@ __global__ void __launch_bounds__(256, MINB) hess34_kernel(H34Params p) {
   }
 }
 
+__global__ void __launch_bounds__(256) hess34_zero(int m, int n, double *Z, WsHeader *hdr) {
+  if (plan_is_stale(&hdr->status, m, n, 0, kHessian34Tag, kHessian34Tag)) return;
+  for (int e = blockIdx.x * 1024 + threadIdx.x; e < min(n * n, (int)(blockIdx.x + 1) * 1024); e += 256) Z[e] = 0.0;
+}
+
 // H = w (Z + Z^T), w = M' / (m (m - 1)) of the general entry
-__global__ void __launch_bounds__(256) hess34_sum(int n, double w, const double *Z, double *H) {
+__global__ void __launch_bounds__(256) hess34_sum(int m, int n, double w, const double *Z, double *H, WsHeader *hdr) {
+  if (plan_is_stale(&hdr->status, m, n, 0, kHessian34Tag, kHessian34Tag)) return;
   __shared__ double t[32][33];
   const int r0 = 32 * blockIdx.y, s0 = 32 * blockIdx.x, x = threadIdx.x & 31;
   for (int y = threadIdx.x >> 5; y < 32; y += 8)
@@ -316,7 +324,7 @@ static int launch_h34(H34Params &p, int sms, cudaStream_t st) {
   return TK_OK;
 }
 
-int hessian34(int m, int n, int storage, const void *K, const double *alpha, double *H, double *Z, cudaStream_t st) {
+int hessian34(int m, int n, int storage, const void *K, const double *alpha, double *H, void *work, cudaStream_t st) {
   DevInfo di;
   int rc = dev_info(&di);
   if (rc != TK_OK) return rc;
@@ -324,7 +332,12 @@ int hessian34(int m, int n, int storage, const void *K, const double *alpha, dou
   p.n = n;
   p.K = reinterpret_cast<const unsigned char *>(K);
   p.alpha = alpha;
-  p.Z = Z;
+  p.hdr = reinterpret_cast<WsHeader *>(work);
+  p.Z = reinterpret_cast<double *>(p.hdr + 1);
+  rc = claim_workspace(m, n, kHessian34Tag, work, st);
+  if (rc != TK_OK) return rc;
+  hess34_zero<<<(unsigned)((n * n + 1023) / 1024), 256, 0, st>>>(m, n, p.Z, p.hdr);
+  TK_CUDA_CHECK(cudaGetLastError());
   if (m == 3) {
     if (storage == TK_F64) rc = launch_h34<double, double, 3, 1, 2>(p, di.sms, st);
     else if (storage == TK_F32) rc = launch_h34<float, float, 3, 1, 4>(p, di.sms, st);
@@ -336,7 +349,7 @@ int hessian34(int m, int n, int storage, const void *K, const double *alpha, dou
   }
   if (rc != TK_OK) return rc;
   const unsigned g = (unsigned)((n + 31) / 32);
-  hess34_sum<<<dim3(g, g), 256, 0, st>>>(n, m == 4 ? 2.0 : 1.0, Z, H);
+  hess34_sum<<<dim3(g, g), 256, 0, st>>>(m, n, m == 4 ? 2.0 : 1.0, p.Z, H, p.hdr);
   TK_CUDA_CHECK(cudaGetLastError());
   return TK_OK;
 }

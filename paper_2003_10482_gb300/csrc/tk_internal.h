@@ -69,6 +69,12 @@ void build_plan(int m, int n, int64_t lo, int64_t hi, int pieces, int64_t row_co
 // header) and record the plan's key in the header.
 int plan_to_device(int m, int n, int64_t lo, int64_t hi, int pieces, int row_cost, int tri_cost, void *work,
                    cudaStream_t st);
+// Make the workspace a pass's own that keeps no plan in it: void the others' plans
+// and set the header's key to (m, n, 0 pieces, [tag, tag)), tag < 0.  Nothing is
+// done when the workspace is the pass's already, so that a captured launch of it
+// replayed over another pass's plan finds a foreign key and does nothing.
+int claim_workspace(int m, int n, int64_t tag, void *work, cudaStream_t st);
+constexpr int64_t kHessian34Tag = -3, kPairsTag = -4;
 // Drop the host's record of which plan the workspace at `work` holds (the
 // memory is about to hold something else, or is new memory at an address a
 // workspace used before).
@@ -112,8 +118,8 @@ size_t build_tc_workspace_bytes(int m, int n, int d);
 int build_tc(int m, int n, int d, const double *X, int feat, int degree, int storage, int64_t off_lo, int64_t off_hi,
              void *K, void *work, size_t work_bytes, cudaStream_t st);
 int build_tc_status(cudaStream_t st);
-// Full Hessian pass at orders 3 and 4; Z: n x n zeroed FP64 values.
-int hessian34(int m, int n, int storage, const void *K, const double *alpha, double *H, double *Z, cudaStream_t st);
+// Full Hessian pass at orders 3 and 4; work: header and n x n FP64 values.
+int hessian34(int m, int n, int storage, const void *K, const double *alpha, double *H, void *work, cudaStream_t st);
 extern int g_build_tc_mode;  // 0: where it pays, 1: always (FP32/BF16), -1: never
 extern tk_batched_config g_batched_cfg;
 // resolved batched launch shape; returns false when the kernel does not cover it
@@ -163,6 +169,8 @@ struct ContractArgs {
 
 // Launch the main pass; the partial sums land in args.part (layout
 // part[block][vec][n + 2]: vec 0 = value, vec 1 = derivative; entry n = S).
+// (contract_plan: its plan alone, of which it returns the pieces)
+int contract_plan(const ContractArgs &a, int *pieces, cudaStream_t st);
 int contract_pass(const ContractArgs &a, int *grid_out, const double **part_out, cudaStream_t st);
 
 // The same pass (FP32/BF16 storage, whole tensor, larger sizes) over the tensor as
