@@ -186,13 +186,20 @@ static int contract_impl(int m, int64_t n, int storage, const void *K, int64_t o
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int vs = vec_dtype == TK_F64 ? 8 : 4;
   unsigned char *wsb = reinterpret_cast<unsigned char *>(work);
-  // One pass for the whole batch when the batched kernel covers the shape and
+  // One pass for the whole batch when a batched kernel covers the shape and
   // the batch is large enough to pay for it: its launch costs about as much
-  // for one vector as for 64 (32 for the HVP), while the single-vector kernel
-  // runs at the HBM rate (measured on GB300, m = 4, n = 300: the batched
-  // kernel wins from B = 28 for K[a^{m-1}] and from B = 16 for the HVP).
-  if ((B >= batched_min_batch(r == m - 2) || rows_pays(m, (int)n, storage, r == m - 2, B, off_lo, off_hi)) &&
-      storage != TK_F64) {
+  // for one vector as for 64 (32 for the HVP), while a single vector's pass
+  // runs at the HBM rate.  Against the streaming pass the column-split kernel
+  // wins from B = 28 for K[a^{m-1}] and from B = 16 for the HVP (m = 4, n = 300);
+  // against the pairs pass it does not win (m = 4, B = 32: n = 300 11.4 / 10.3 ms
+  // against 7.9 / 9.2, n = 400 21.4 / 24.5 against the same), so there only the
+  // rows and tensor-core passes are taken, from the batch at which they pay.
+  const bool dual = r == m - 2;
+  const bool singles = g_batched_cfg.min_batch == 0 && g_batched_cfg.tensor_cores == 0 &&
+                       pairs_covers(m, (int)n, storage, off_lo, off_hi) && work_bytes >= pairs_workspace_bytes((int)n);
+  if (storage != TK_F64 && (rows_pays(m, (int)n, storage, dual, B, off_lo, off_hi) ||
+                            (B >= batched_min_batch(dual) &&
+                             !(singles && !tc_covers(m, (int)n, storage, dual, B, off_lo, off_hi))))) {
     BatchedArgs ba;
     memset(&ba, 0, sizeof(ba));
     ba.m = m;
@@ -209,16 +216,18 @@ static int contract_impl(int m, int64_t n, int storage, const void *K, int64_t o
     ba.S = (r == m - 1) ? S : nullptr;
     ba.work = work;
     ba.work_bytes = work_bytes;
-    if (tc_covers(m, (int)n, storage, r == m - 2, B, off_lo, off_hi)) {
+    if (tc_covers(m, (int)n, storage, dual, B, off_lo, off_hi)) {
       rc = contract_batched_tc(ba, st);
       if (rc != TK_EUNSUPPORTED) return rc;
     }
-    if (rows_covers(m, (int)n, storage, r == m - 2, B, off_lo, off_hi)) {
+    if (rows_covers(m, (int)n, storage, dual, B, off_lo, off_hi)) {
       rc = contract_batched_rows(ba, st);
       if (rc != TK_EUNSUPPORTED) return rc;
     }
-    rc = contract_batched(ba, st);
-    if (rc != TK_EUNSUPPORTED) return rc;
+    if (B >= batched_min_batch(dual)) {
+      rc = contract_batched(ba, st);
+      if (rc != TK_EUNSUPPORTED) return rc;
+    }
   }
   for (int64_t b = 0; b < B; ++b) {
     ContractArgs a;

@@ -636,6 +636,15 @@ size_t tc_workspace_bytes(int m, int n, int64_t B, int sms) {
   return tc_layout(n, B, sms, nj, nt).total;
 }
 
+static bool tc_plan_current(int m, int n, int P, void *work) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::lock_guard<std::mutex> lk(g_tcmu);
+  const TcKey key{m, n, P};
+  auto up = g_tcup.find({dev, work});
+  return up != g_tcup.end() && !(up->second < key) && !(key < up->second);
+}
+
 // Make sure the workspace holds the jobs, triangles and job ranges of (m, n, P).
 static int tc_upload_plan(int m, int n, int P, size_t njobs, size_t ntris, const TcLayout &L, void *work,
                           cudaStream_t st) {
@@ -787,13 +796,16 @@ bool rows_covers(int m, int n, int storage, bool dual, int64_t B, int64_t off_lo
 }
 
 // The pass costs the same for 1 to 32 vectors (64 of the contraction); single
-// passes reach that at some n/16 (n/12) of them.  Measured, the pass against one
-// single pass (m = 4 FP32, Hessian-vector / contraction): n = 64 118 / 148 us
-// against 29 / 29, n = 100 0.28 / 0.39 ms against 0.041 / 0.042, n = 150 0.73 / 0.95
-// against 0.079 / 0.071, n = 300 6.9 / 8.8 against 0.49 / 0.36.
+// streaming passes reach that at some n/16 (n/12) of them, the pairs passes of
+// m = 4, n >= 200 at n/14 (n/9).  Measured, the pass against one single pass (m = 4
+// FP32, Hessian-vector / contraction): n = 64 118 / 148 us against 29 / 29, n = 100
+// 0.28 / 0.39 ms against 0.041 / 0.042, n = 150 0.73 / 0.95 against 0.079 / 0.071,
+// n = 200 1.9 / 2.5 against 0.17 / 0.12, n = 250 3.5 / 4.8 against 0.22 / 0.16,
+// n = 300 6.9 / 8.8 against 0.29 / 0.25 (BF16 7.5 / 10.1 against 0.29 / 0.21).
 bool rows_pays(int m, int n, int storage, bool dual, int64_t B, int64_t off_lo, int64_t off_hi) {
+  const bool pairs = pairs_covers(m, n, storage, off_lo, off_hi);
   return g_batched_cfg.min_batch == 0 && rows_covers(m, n, storage, dual, B, off_lo, off_hi) &&
-         B * (dual ? 16 : 12) >= n;
+         B * (pairs ? (dual ? 14 : 9) : (dual ? 16 : 12)) >= n;
 }
 
 size_t rows_workspace_bytes(int m, int n, int64_t B, int sms) {
@@ -827,6 +839,12 @@ int contract_batched_rows(const BatchedArgs &a, cudaStream_t st) {
   if (a.work_bytes < L.total || rg_smem<128>(nkc) > (size_t)di.smem_optin)
     return fail(TK_EUNSUPPORTED, "batched rows pass: workspace or shared memory");
   unsigned char *ws = reinterpret_cast<unsigned char *>(a.work);
+  // the upload waits for its copy, which a stream capture does not allow: the
+  // passes that need no such wait are recorded instead
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  TK_CUDA_CHECK(cudaStreamIsCapturing(st, &cs));
+  if (cs != cudaStreamCaptureStatusNone && !tc_plan_current(m, n, sh.P, a.work))
+    return fail(TK_EUNSUPPORTED, "batched rows pass: no plan in the workspace under stream capture");
   rc = tc_upload_plan(m, n, sh.P, njobs, ntris, L.t, a.work, st);
   if (rc != TK_OK) return rc;
   RgParams p;
