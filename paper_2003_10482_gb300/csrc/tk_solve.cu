@@ -443,8 +443,9 @@ extern "C" int tk_solve_dual(const tk_problem *P, const tk_solve_opts *O, double
     s.hws = base + L.hws;
     // this region's offset in the workspace depends on B: a plan recorded
     // here by an earlier call may have been overwritten since (by that call's
-    // matrices at another B), so the pass uploads its plan afresh
+    // matrices at another B), so the pass uploads its plan (writes its key) afresh
     forget_hessian_plan(s.hws);
+    forget_plan(s.hws);
     s.hws_bytes = L.hcur - L.hws;
     Hcur = reinterpret_cast<double *>(base + L.hcur);
     Htrial = reinterpret_cast<double *>(base + L.htrial);

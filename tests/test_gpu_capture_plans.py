@@ -70,3 +70,21 @@ def test_batched_rows_first_call_under_capture():
     assert tk.tk_status_read(work) == tk.TK_OK
     assert torch.equal(G[0], one.reshape(-1))  # the single-vector pass
     assert torch.allclose(G, rows, rtol=0, atol=1e-5 * float(rows.abs().max()))
+
+
+def test_solves_of_changing_sizes_share_a_workspace():
+    """A solve's Hessian region moves with its sizes, over what an earlier solve kept there."""
+    K = {n: build(4, n) for n in (30, 64, 130)}
+    y = {n: torch.tensor(synth.alpha_like(n, salt=1304), device="cuda") for n in K}
+
+    def solve(n, B):
+        lam = torch.linspace(0.8, 1.2, B, dtype=torch.float64, device="cuda")
+        return tk.tk_solve_dual(K[n], 4, n, y[n], lam, method="newton_full", tol=0.0, rel_gap=1e-9, max_iter=30)[0]
+
+    tk._solve_ws.clear()
+    order = [(130, 8), (64, 1), (30, 8), (130, 1), (64, 8), (64, 2), (30, 2), (130, 4), (64, 4)]
+    first = {c: solve(*c).clone() for c in order}
+    for c in order[::-1] + order:
+        again = solve(*c)
+        # the FP64 sums of the Hessian pass may differ in the last bits
+        assert torch.allclose(again, first[c], rtol=0, atol=1e-6 * float(first[c].abs().max())), c
