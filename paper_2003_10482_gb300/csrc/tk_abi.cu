@@ -192,7 +192,7 @@ static int contract_impl(int m, int64_t n, int storage, const void *K, int64_t o
   // runs at the HBM rate.  Against the streaming pass the column-split kernel
   // wins from B = 28 for K[a^{m-1}] and from B = 16 for the HVP (m = 4, n = 300);
   // against the pairs pass it does not win (m = 4, B = 32: n = 300 11.4 / 10.3 ms
-  // against 7.9 / 9.2, n = 400 21.4 / 24.5 against the same), so there only the
+  // against 7.9 / 8.8, n = 400 21.4 against 21.8), so there only the
   // rows and tensor-core passes are taken, from the batch at which they pay.
   const bool dual = r == m - 2;
   const bool singles = g_batched_cfg.min_batch == 0 && g_batched_cfg.tensor_cores == 0 &&

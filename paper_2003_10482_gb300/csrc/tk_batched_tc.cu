@@ -800,8 +800,8 @@ bool rows_covers(int m, int n, int storage, bool dual, int64_t B, int64_t off_lo
 // m = 4, n >= 200 at n/14 (n/9).  Measured, the pass against one single pass (m = 4
 // FP32, Hessian-vector / contraction): n = 64 118 / 148 us against 29 / 29, n = 100
 // 0.28 / 0.39 ms against 0.041 / 0.042, n = 150 0.73 / 0.95 against 0.079 / 0.071,
-// n = 200 1.9 / 2.5 against 0.17 / 0.12, n = 250 3.5 / 4.8 against 0.22 / 0.16,
-// n = 300 6.9 / 8.8 against 0.29 / 0.25 (BF16 7.5 / 10.1 against 0.29 / 0.21).
+// n = 200 1.9 / 2.5 against 0.15 / 0.11, n = 250 3.5 / 4.8 against 0.19 / 0.16,
+// n = 300 6.9 / 8.8 against 0.28 / 0.25 (BF16 7.5 / 10.1 against 0.24 / 0.17).
 bool rows_pays(int m, int n, int storage, bool dual, int64_t B, int64_t off_lo, int64_t off_hi) {
   const bool pairs = pairs_covers(m, n, storage, off_lo, off_hi);
   return g_batched_cfg.min_batch == 0 && rows_covers(m, n, storage, dual, B, off_lo, off_hi) &&

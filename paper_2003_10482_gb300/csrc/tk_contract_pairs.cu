@@ -19,26 +19,29 @@
 // product), with no triangles and no per-row work inside the loop: a warp holds one
 // tile of 512 pairs of one b -- Y and z_p = f a_c a_d in registers, 16 of each a
 // lane -- and walks the prefixes i = 0..b, one bulk copy of 2 KB (1 KB for BF16)
-// each into a ring of 10 KB.  Eight prefixes' row sums are reduced over the
-// lanes together (9 shuffles).  Every Y_b[p] and every (Q, tile) row sum belongs to
-// one warp: plain stores, no atomics, sums in a fixed order.  Two small kernels add
-// up Y over b, tau over the tiles (FP64) and form g, S and the objective.
+// each into a ring of 8 KB.  Eight prefixes' row sums are reduced over the
+// lanes together (9 shuffles); the eight are unrolled, so that their ring slots are
+// constants, and two multiply-adds are one fma.rn.f32x2 (the same roundings).  Every
+// Y_b[p] and every (Q, tile) row sum belongs to one warp: plain stores, no atomics,
+// sums in a fixed order.  Two small kernels add up Y over b, tau over the tiles
+// (FP64) and form g, S and the objective.
 //
-// What bounds it: the contraction of FP32 storage HBM (the main kernel reads
-// 7.2 TB/s at n = 400, issue 45 % busy); the product and BF16 storage the per-prefix
-// work, some 3 to 4.4 prefix tiles per ns over the chip (110 to 170 instructions
-// each, 16 warps an SM held by Y, z and the ring).  Measured, streaming pass ->
-// this one: FP32 contraction n = 400 885 -> 685 us (objective call 874 -> 677),
-// n = 300 399 -> 264, n = 250 238 -> 177, n = 200 162 -> 141; Hessian-vector product
-// n = 400 1037 -> 775, n = 351 701 -> 499, n = 250 276 -> 237, n = 200 188 -> 192 (below,
-// the four launches cost more than they save); BF16 n = 600 2852 -> 2424, its product
-// 3616 -> 3547, n = 400 741 -> 548 and 958 -> 788.  Loads into registers instead of
+// What bounds it: HBM for FP32 storage at n = 400 (the main kernel reads 7.2 TB/s,
+// issue 45 % busy); the per-prefix work for BF16 storage and smaller n (16 warps an SM
+// held by Y, z and the ring), and below n = 250 the longest walk of one warp, n
+// prefixes.  Measured, streaming pass -> this one: FP32 contraction n = 400 866 -> 680
+// us, n = 300 387 -> 251, n = 250 225 -> 155, n = 200 148 -> 114; Hessian-vector product
+// n = 400 1026 -> 719, n = 351 688 -> 456, n = 250 262 -> 194, n = 200 174 -> 150; BF16
+// n = 600 2836 -> 2069, its product 3599 -> 2323, n = 400 729 -> 431 and 945 -> 558, n = 200
+// 145 -> 110 and 164 -> 152.  With a ring of 10 KB, slots counted at run time and single
+// multiply-adds BF16 n = 600 took 2424 and 3547 us.  Loads into registers instead of
 // the ring (1 KB or 2 KB a prefix, one to four in flight) read 4.4 to 4.7 TB/s; the
 // same walk over b for a fixed i 3.7.
 #include <cuda_bf16.h>
 #include <stddef.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "tk_prefix.cuh"
 
@@ -46,9 +49,9 @@ namespace tk {
 
 constexpr int kPT = 512;        // pairs per tile
 constexpr int kPC = kPT / 32;   // of them a lane's
-// prefixes in flight a warp: 10 KB, 160 an SM
+// prefixes in flight a warp: 8 KB, 128 an SM (a power of two: constant slots)
 template <typename ST>
-constexpr int kPNB = sizeof(ST) == 4 ? 5 : 10;
+constexpr int kPNB = sizeof(ST) == 4 ? 4 : 8;
 constexpr int kPRow = 8;        // prefixes whose row sums are reduced together
 constexpr int kPMinN = 200;     // points from which the pass is taken (see the figures above)
 constexpr int kPMaxN = 640;     // and to which (its sums take up to 5 % of the tensor's bytes)
@@ -130,76 +133,105 @@ __global__ void __launch_bounds__(256, 2) pairs_kernel(PParams p) {
   const int p0 = t * kPT + lane, count = min(kPT, np - t * kPT);
   const ST *K = reinterpret_cast<const ST *>(p.K) + (int)(multiset(n, 3) - multiset(L, 3)) + t * kPT;
 
-  float z[kPC], zd[kPC], Y[kPC], Yd[kPC];
+  float2 z[kPC / 2], zd[kPC / 2], Y[kPC / 2], Yd[kPC / 2];  // pairs lane + 32 k of the tile, k even and odd
   {
     const float *zp = p.z + pair_start(n, b) + p0, *zdp = p.zd + pair_start(n, b) + p0;
-#pragma unroll
-    for (int k = 0; k < kPC; ++k) {
+    auto ldz = [&](const float *v, int k) -> float {
       const int q = p0 + 32 * k;
       const float f = q == 0 ? 1.f / 3.f : q < L ? 0.5f : 1.f;  // the row c = b at kb = 1
-      z[k] = q < np ? f * zp[32 * k] : 0.f;
-      zd[k] = D && q < np ? f * zdp[32 * k] : 0.f;
-      Y[k] = Yd[k] = 0.f;
+      return q < np ? f * v[32 * k] : 0.f;
+    };
+#pragma unroll
+    for (int j = 0; j < kPC / 2; ++j) {
+      z[j] = make_float2(ldz(zp, 2 * j), ldz(zp, 2 * j + 1));
+      zd[j] = D ? make_float2(ldz(zdp, 2 * j), ldz(zdp, 2 * j + 1)) : make_float2(0.f, 0.f);
+      Y[j] = Yd[j] = make_float2(0.f, 0.f);
     }
   }
   const float ab = 6.f * a_s[b], vb = D ? 6.f * v_s[b] : 0.f;
   float *tp = p.t + (size_t)item * n, *tdp = p.td + (size_t)item * n;
-  for (int i = 0; i < min(NB, b + 1); ++i) ring.issue(i, K + slab[i], count);
-  int slot = 0;
-  uint32_t phase = 0;
-  bool ok = true;
-  for (int i0 = 0; i0 <= b && ok; i0 += kPRow) {
-    float s[kPRow], sd[kPRow];
+  // one prefix: columns into Y, the lane's part of the row sums
+  auto add = [&](const float2 (&x)[kPC / 2], float ca, float cd, float *s, float *sd) {
+    float2 s2 = make_float2(0.f, 0.f), d2 = s2;
+    const float2 c2 = make_float2(ca, ca), e2 = make_float2(cd, cd);
 #pragma unroll
-    for (int r = 0; r < kPRow; ++r) {
-      s[r] = sd[r] = 0.f;
-      const int i = i0 + r;
-      if (i <= b && ok) {
-        const ST *xp = ring.take(slot, phase, K + slab[i], &ok) + lane;
-        float x[kPC];
-        if (count == kPT) {
-#pragma unroll
-          for (int k = 0; k < kPC; ++k) x[k] = ld_elem<ST, float>(xp + 32 * k);
-        } else {
-#pragma unroll
-          for (int k = 0; k < kPC; ++k) x[k] = lane + 32 * k < count ? ld_elem<ST, float>(xp + 32 * k) : 0.f;
-        }
-        if (i + NB <= b) ring.issue(slot, K + slab[i + NB], count);
-        if (++slot == NB) {
-          slot = 0;
-          phase ^= 1u;
-        }
-        float ca = ab * a_s[i], cd = D ? vb * a_s[i] + ab * v_s[i] : 0.f;
-        if (i == b) {
-          // Q = (b, b): M' is half, and the row c = b has kb = 2 (f = 1/3, 1/12)
-          ca *= 0.5f;
-          cd *= 0.5f;
-#pragma unroll
-          for (int k = 0; k < kPC; ++k) {
-            const int q = p0 + 32 * k;
-            if (q < L) x[k] *= q == 0 ? 0.5f : 2.f / 3.f;
-          }
-        }
-        float s0 = 0.f, s1 = 0.f, d0 = 0.f, d1 = 0.f;
-#pragma unroll
-        for (int k = 0; k < kPC; ++k) {
-          Y[k] = __fmaf_rn(ca, x[k], Y[k]);
-          if (k & 1) s1 = __fmaf_rn(z[k], x[k], s1); else s0 = __fmaf_rn(z[k], x[k], s0);
-          if (D) {
-            Yd[k] = __fmaf_rn(cd, x[k], Yd[k]);
-            if (k & 1) d1 = __fmaf_rn(zd[k], x[k], d1); else d0 = __fmaf_rn(zd[k], x[k], d0);
-          }
-        }
-        s[r] = s0 + s1;
-        if (D) sd[r] = d0 + d1;
+    for (int j = 0; j < kPC / 2; ++j) {
+      Y[j] = fma2(c2, x[j], Y[j]);
+      s2 = fma2(z[j], x[j], s2);
+      if (D) {
+        Yd[j] = fma2(e2, x[j], Yd[j]);
+        d2 = fma2(zd[j], x[j], d2);
       }
     }
-    const float v = warp_scatter8(s, lane);
-    const int i = i0 + (lane >> 2);
-    if ((lane & 3) == 0 && i <= b) tp[i] = v;
-    if (D) {
-      const float vd = warp_scatter8(sd, lane);
-      if ((lane & 3) == 0 && i <= b) tdp[i] = vd;
+    *s = s2.x + s2.y;
+    if (D) *sd = d2.x + d2.y;
+  };
+  for (int i = 0; i < min(NB, b + 1); ++i) ring.issue(i, K + slab[i], count);
+  bool ok = true;
+  int i0 = 0, fail_at = 0;
+  // groups of 8 prefixes below b, whose ring slots are constants (a whole tile's
+  // segment is never the array's last)
+  auto groups = [&](auto whole) {
+    constexpr bool kWhole = decltype(whole)::value;
+    auto ld = [&](const ST *xp, int k) -> float {
+      return kWhole || lane + 32 * k < count ? ld_elem<ST, float>(xp + 32 * k) : 0.f;
+    };
+    for (; i0 + kPRow <= b && ok; i0 += kPRow) {
+      float s[kPRow], sd[kPRow];
+#pragma unroll
+      for (int r = 0; r < kPRow; ++r) {
+        const int i = i0 + r;
+        bool landed;
+        const ST *xp = ring.take(r % NB, (uint32_t)(i / NB) & 1u, K + slab[i], &landed) + lane;
+        if (!landed && ok) {
+          ok = false;
+          fail_at = i;
+        }
+        float2 x[kPC / 2];
+#pragma unroll
+        for (int j = 0; j < kPC / 2; ++j) x[j] = make_float2(ld(xp, 2 * j), ld(xp, 2 * j + 1));
+        if (i + NB <= b && ok) ring.template issue<!kWhole>(r % NB, K + slab[i + NB], kWhole ? kPT : count);
+        add(x, ab * a_s[i], D ? vb * a_s[i] + ab * v_s[i] : 0.f, &s[r], &sd[r]);
+      }
+      const float v = warp_scatter8(s, lane);
+      if ((lane & 3) == 0) tp[i0 + (lane >> 2)] = v;
+      if (D) {
+        const float vd = warp_scatter8(sd, lane);
+        if ((lane & 3) == 0) tdp[i0 + (lane >> 2)] = vd;
+      }
+    }
+  };
+  if (count == kPT) groups(std::true_type());
+  else groups(std::false_type());
+  // the others, one by one
+#pragma unroll 1
+  for (; i0 <= b && ok; ++i0) {
+    const ST *xp = ring.take(i0 & (NB - 1), (uint32_t)(i0 / NB) & 1u, K + slab[i0], &ok) + lane;
+    float2 x[kPC / 2];
+#pragma unroll
+    for (int k = 0; k < kPC; ++k) {
+      float e = lane + 32 * k < count ? ld_elem<ST, float>(xp + 32 * k) : 0.f;
+      // Q = (b, b): M' is half, and the row c = b has kb = 2 (f = 1/3, 1/12)
+      const int q = p0 + 32 * k;
+      if (i0 == b && q < L) e *= q == 0 ? 0.5f : 2.f / 3.f;
+      if (k & 1) x[k / 2].y = e; else x[k / 2].x = e;
+    }
+    if (!ok) {
+      fail_at = i0;
+      break;
+    }
+    if (i0 + NB <= b) ring.issue(i0 & (NB - 1), K + slab[i0 + NB], count);
+    const float h = i0 == b ? 0.5f : 1.f;
+    float s = 0.f, sd = 0.f;
+    add(x, h * (ab * a_s[i0]), D ? h * (vb * a_s[i0] + ab * v_s[i0]) : 0.f, &s, &sd);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (D) sd += __shfl_xor_sync(0xffffffffu, sd, o);
+    }
+    if (lane == 0) {
+      tp[i0] = s;
+      if (D) tdp[i0] = sd;
     }
   }
   if (!ok) {
@@ -207,7 +239,7 @@ __global__ void __launch_bounds__(256, 2) pairs_kernel(PParams p) {
       atomicExch(&p.hdr->status, TK_ETIMEOUT);
       p.hdr->where = kSiteContractWait;
     }
-    ring.drain(slot, phase);
+    ring.drain_from(fail_at, b);
   }
   // the row weights at kb = 1 (c = d is weighted with y)
   float *yp = p.Y + (size_t)item * kPT + lane, *ydp = p.Yd + (size_t)item * kPT + lane;
@@ -215,8 +247,8 @@ __global__ void __launch_bounds__(256, 2) pairs_kernel(PParams p) {
   for (int k = 0; k < kPC; ++k) {
     const int q = p0 + 32 * k;
     const float f = q == 0 ? 1.f / 3.f : q < L ? 0.5f : 1.f;
-    yp[32 * k] = f * Y[k];
-    if (D) ydp[32 * k] = f * Yd[k];
+    yp[32 * k] = f * (k & 1 ? Y[k / 2].y : Y[k / 2].x);
+    if (D) ydp[32 * k] = f * (k & 1 ? Yd[k / 2].y : Yd[k / 2].x);
   }
 }
 

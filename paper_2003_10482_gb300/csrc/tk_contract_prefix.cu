@@ -17,16 +17,17 @@
 //
 // A warp holds a tile of 256 pairs of one b (Y and z_p = f a_c a_d of kb = 1, 8 of
 // each a lane) and walks a run of prefixes, one load and two multiply-adds per
-// entry, one bulk copy per prefix into a ring of six.  A prefix's offset is a sum of m - 3 table
+// entry, one bulk copy per prefix into a ring of four.  A prefix's offset is a sum of m - 3 table
 // values,  base(Q) = C(n+m-1, m) - sum_j W_j[q_j] - C(n-b+2, 3),
 // W_j[x] = C(n-1-x + m-j-1, m-j), its index in tau likewise; 32 lanes form the
 // next 32 prefixes' offsets and coefficients together.  Plain stores, fixed order.
 //
 // What bounds it: the work per (prefix, tile) -- its copy's issue and wait, the
 // broadcasts of its record -- at some 150 entries each.  Measured, streaming pass ->
-// this one: m = 6, n = 80 1970 -> 1266 us (1.75 GB), n = 60 584 -> 461, BF16 n = 80
-// 2026 -> 1277; m = 5, n = 100 333 -> 290.  At m = 6, n = 45 the six launches took 254
-// against 201 us: hence kXMinEntries.
+// this one: m = 6, n = 80 1970 -> 1158 us (1.75 GB; 1266 with slots counted at run time
+// and single multiply-adds), n = 60 584 -> 438, BF16 n = 80 2026 -> 1189; m = 5, n = 100
+// 333 -> 277.  At m = 6, n = 45 the six launches took 254 against 201 us: hence
+// kXMinEntries.
 #include <cuda_bf16.h>
 #include <stddef.h>
 
@@ -38,7 +39,7 @@ namespace tk {
 
 constexpr int kXC = 8;              // chunks of 32 pairs per tile
 constexpr int kXT = 32 * kXC;
-constexpr int kXNB = 6;             // prefixes in flight a warp
+constexpr int kXNB = 4;             // prefixes in flight a warp (divides 8: constant slots)
 constexpr int kXSlices = 32;        // slices of b in the sums of y
 constexpr int kXMaxN = 256;
 constexpr int64_t kXMinEntries = 50000000;  // entries from which the pass is taken
@@ -116,12 +117,15 @@ __global__ void __launch_bounds__(256, 3) prefix_kernel(XParams p) {
   const int sp = (item - p.item[b]) / nt, t = item - p.item[b] - sp * nt;
   const int L = n - b, np = L * (L + 1) / 2, p0 = t * kXT + lane;
   const bool first_row = t * kXT < L;
-  float z[kXC], Y[kXC];
-#pragma unroll
-  for (int k = 0; k < kXC; ++k) {
+  float2 z[kXC / 2], Y[kXC / 2];  // pairs lane + 32 k of the tile, k even and odd
+  auto ldz = [&](int k) -> float {
     const int q = p0 + 32 * k;
-    z[k] = q < np ? p.z[pair_start(n, b) + q] * (q == 0 ? 1.f / 3.f : q < L ? 0.5f : 1.f) : 0.f;
-    Y[k] = 0.f;
+    return q < np ? p.z[pair_start(n, b) + q] * (q == 0 ? 1.f / 3.f : q < L ? 0.5f : 1.f) : 0.f;
+  };
+#pragma unroll
+  for (int j = 0; j < kXC / 2; ++j) {
+    z[j] = make_float2(ldz(2 * j), ldz(2 * j + 1));
+    Y[j] = make_float2(0.f, 0.f);
   }
   const ST *K = reinterpret_cast<const ST *>(p.K) + (p.size - multiset(n - b, 3)) + t * kXT;
   float *tp = p.t + (size_t)t * p.nq + (p.nq - (n - b));
@@ -193,12 +197,11 @@ __global__ void __launch_bounds__(256, 3) prefix_kernel(XParams p) {
     rec.cnt = cnt;
   };
   const int count = min(kXT, np - t * kXT);
-  int slot = 0;  // of the next segment
-  uint32_t phase = 0;
+  int fail_at = 0;  // segment (mod 8) whose copy did not land
   bool ok = true;
   fill(cur);
   fill(nxt);
-  // (a batch that another one follows is full, and longer than the ring)
+  // (a batch that another one follows is full: segment i of any batch is in slot i % kXNB)
   for (int i = 0; i < min(kXNB, cur.cnt); ++i) ring.issue(i, K + __shfl_sync(0xffffffffu, cur.off, i), count);
   while (cur.cnt > 0 && ok) {
     const int cnt = cur.cnt;
@@ -210,7 +213,8 @@ __global__ void __launch_bounds__(256, 3) prefix_kernel(XParams p) {
         const int i = r0 + r;
         s[r] = 0.f;
         if (i < cnt && ok) {
-          const ST *xp = ring.take(slot, phase, K + __shfl_sync(0xffffffffu, cur.off, i), &ok) + lane;
+          const ST *xp = ring.take(r % kXNB, (uint32_t)(r / kXNB) & 1u, K + __shfl_sync(0xffffffffu, cur.off, i), &ok) + lane;
+          if (!ok) fail_at = r;
           float x[kXC];
           if (count == kXT) {
 #pragma unroll
@@ -221,11 +225,7 @@ __global__ void __launch_bounds__(256, 3) prefix_kernel(XParams p) {
           }
           // the slot takes the prefix kXNB further on, of this batch or the next
           const int f = i + kXNB - cnt;
-          if (f < nxt.cnt) ring.issue(slot, K + __shfl_sync(0xffffffffu, f < 0 ? cur.off : nxt.off, f < 0 ? f + cnt : f), count);
-          if (++slot == kXNB) {
-            slot = 0;
-            phase ^= 1u;
-          }
+          if (f < nxt.cnt && ok) ring.issue(r % kXNB, K + __shfl_sync(0xffffffffu, f < 0 ? cur.off : nxt.off, f < 0 ? f + cnt : f), count);
           const float ca = __shfl_sync(0xffffffffu, cur.coef, i);
           if (first_row && (multi >> i & 1)) {
             const float k1 = (float)__shfl_sync(0xffffffffu, cur.kb, i);
@@ -236,13 +236,15 @@ __global__ void __launch_bounds__(256, 3) prefix_kernel(XParams p) {
               if (q < L) x[k] *= q == 0 ? w0 : w1;
             }
           }
-          float s0 = 0.f, s1 = 0.f;
+          const float2 c2 = make_float2(ca, ca);
+          float2 s2 = make_float2(0.f, 0.f);
 #pragma unroll
-          for (int k = 0; k < kXC; ++k) {
-            Y[k] = __fmaf_rn(ca, x[k], Y[k]);
-            if (k & 1) s1 = __fmaf_rn(z[k], x[k], s1); else s0 = __fmaf_rn(z[k], x[k], s0);
+          for (int j = 0; j < kXC / 2; ++j) {
+            const float2 x2 = make_float2(x[2 * j], x[2 * j + 1]);
+            Y[j] = fma2(c2, x2, Y[j]);
+            s2 = fma2(z[j], x2, s2);
           }
-          s[r] = s0 + s1;
+          s[r] = s2.x + s2.y;
         }
       }
       const float v = warp_scatter8(s, lane);
@@ -257,13 +259,13 @@ __global__ void __launch_bounds__(256, 3) prefix_kernel(XParams p) {
       atomicExch(&p.hdr->status, TK_ETIMEOUT);
       p.hdr->where = kSiteContractWait;
     }
-    ring.drain(slot, phase);
+    ring.drain(fail_at % kXNB, (uint32_t)(fail_at / kXNB) & 1u);
   }
   float *yp = p.Y + (size_t)item * kXT + lane;
 #pragma unroll
   for (int k = 0; k < kXC; ++k) {
     const int q = p0 + 32 * k;
-    yp[32 * k] = (q == 0 ? 1.f / 3.f : q < L ? 0.5f : 1.f) * Y[k];
+    yp[32 * k] = (q == 0 ? 1.f / 3.f : q < L ? 0.5f : 1.f) * (k & 1 ? Y[k / 2].y : Y[k / 2].x);
   }
 }
 

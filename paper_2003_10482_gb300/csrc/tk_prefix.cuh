@@ -46,16 +46,18 @@ struct RowRing {
   }
   // start the copy of `count` entries at src into slot s (every lane has read the
   // slot's last segment and calls)
+  // (END: the segment may be the array's last)
+  template <bool END = true>
   __device__ __forceinline__ void issue(int s, const ST *src, int count) {
     const unsigned char *p = reinterpret_cast<const unsigned char *>(src);
     const uint32_t lead = (uint32_t)reinterpret_cast<uintptr_t>(p) & 15u;
     uint32_t bytes = (lead + (uint32_t)count * (uint32_t)sizeof(ST) + 15u) & ~15u;
     unsigned char *dst = buf + s * kBytes;
     __syncwarp();
-    if (p - lead + bytes > tail) bytes = by_hand(dst, p - lead, p + (size_t)count * sizeof(ST));
+    if (END && p - lead + bytes > tail) bytes = by_hand(dst, p - lead, p + (size_t)count * sizeof(ST));
     if (lane == 0) {
       fence_proxy_async();
-      if (bytes) {
+      if (!END || bytes) {
         mbar_expect_tx(&bar[s], bytes);
         bulk_g2s(dst, p - lead, bytes, &bar[s]);
       } else {
@@ -76,13 +78,27 @@ struct RowRing {
     *ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[s], phase));
     return reinterpret_cast<const ST *>(buf + s * kBytes + ((uint32_t)reinterpret_cast<uintptr_t>(src) & 15u));
   }
-  // after a wait that ran out: give the copies in flight from slot s on their
-  // time before the block can end
+  // after a wait for segment i (of the walk 0, 1, .. last, NB a power of two) that ran
+  // out: give the copies in flight their time before the block can end
+  __device__ __forceinline__ void drain_from(int i, int last) {
+    for (int j = i; j <= last && j < i + NB; ++j) mbar_wait_bounded(&bar[j & (NB - 1)], (uint32_t)(j / NB) & 1u);
+  }
+  // the same from slot s on
   __device__ __noinline__ void drain(int s, uint32_t phase) {
     for (int k = 0; k < NB; ++k)
       mbar_wait_bounded(&bar[(s + k) % NB], phase ^ (s + k >= NB ? 1u : 0u));
   }
 };
+
+// a * b + c of both halves, each rounded as by __fmaf_rn, in one instruction
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rc;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
+      "fma.rn.f32x2 rc, ra, rb, rc;\n\tmov.b64 {%0, %1}, rc;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
 
 // Sum of the 8 values of every lane over the warp: lane l ends with value l >> 2's
 __device__ __forceinline__ float warp_scatter8(float (&v)[8], int lane) {
