@@ -27,10 +27,10 @@
 // depend on b, nor the distance between the slabs of two i: an address is
 // slab(i) + o(b) - D_r, one 32-bit subtraction and a widening multiply-add away.
 // The 8 warps of a block take neighbouring column chunks of the same rows, so a
-// row segment's shared cache lines are read from HBM once (1.39 GB for 1.38).
+// row segment's shared cache lines are mostly read from HBM once (1.48 GB for 1.38).
 //
 // What bounds it (m = 4, n = 300 FP32): the instructions, some 540 per step of
-// 1024 entries (209 M in all, issue 38 % busy with 16 warps an SM; without the
+// 1024 entries (235 M in all, issue 46 % busy with 16 warps an SM; without the
 // loads it takes the same time, without the atomic additions a tenth less); 128
 // registers hold T (4 i x 8 rows), the loaded entries and R.  0.50 ms against
 // 3.59 for the pass of tk_hessian.cu (947 M instructions, three block barriers
