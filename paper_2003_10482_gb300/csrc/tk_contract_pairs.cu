@@ -193,10 +193,10 @@ __global__ void __launch_bounds__(256, 2) pairs_kernel(PParams p) {
         if (i + NB <= b && ok) ring.template issue<!kWhole>(r % NB, K + slab[i + NB], kWhole ? kPT : count);
         add(x, ab * a_s[i], D ? vb * a_s[i] + ab * v_s[i] : 0.f, &s[r], &sd[r]);
       }
-      const float v = warp_scatter8(s, lane);
+      const float v = warp_scatter(s, lane);
       if ((lane & 3) == 0) tp[i0 + (lane >> 2)] = v;
       if (D) {
-        const float vd = warp_scatter8(sd, lane);
+        const float vd = warp_scatter(sd, lane);
         if ((lane & 3) == 0) tdp[i0 + (lane >> 2)] = vd;
       }
     }

@@ -24,9 +24,10 @@
 //
 // What bounds it: the work per (prefix, tile) -- its copy's issue and wait, the
 // broadcasts of its record -- at some 150 entries each.  Measured, streaming pass ->
-// this one: m = 6, n = 80 1970 -> 1158 us (1.75 GB; 1266 with slots counted at run time
-// and single multiply-adds), n = 60 584 -> 438, BF16 n = 80 2026 -> 1189; m = 5, n = 100
-// 333 -> 277.  At m = 6, n = 45 the six launches took 254 against 201 us: hence
+// this one: m = 6, n = 80 1970 -> 1026 us (1.75 GB; 1266 with slots counted at run time
+// and single multiply-adds; 1153 with eight prefixes unrolled instead of four: 1.9
+// stalls for instructions per issue), n = 60 584 -> 390, BF16 n = 80 2026 -> 1035; m = 5,
+// n = 100 333 -> 254.  At m = 6, n = 45 the six launches took 254 against 201 us: hence
 // kXMinEntries.
 #include <cuda_bf16.h>
 #include <stddef.h>
@@ -39,7 +40,8 @@ namespace tk {
 
 constexpr int kXC = 8;              // chunks of 32 pairs per tile
 constexpr int kXT = 32 * kXC;
-constexpr int kXNB = 4;             // prefixes in flight a warp (divides 8: constant slots)
+constexpr int kXNB = 4;             // prefixes in flight a warp
+constexpr int kXRow = 4;            // prefixes unrolled (a multiple of kXNB: constant slots)
 constexpr int kXSlices = 32;        // slices of b in the sums of y
 constexpr int kXMaxN = 256;
 constexpr int64_t kXMinEntries = 50000000;  // entries from which the pass is taken
@@ -197,7 +199,7 @@ __global__ void __launch_bounds__(256, 3) prefix_kernel(XParams p) {
     rec.cnt = cnt;
   };
   const int count = min(kXT, np - t * kXT);
-  int fail_at = 0;  // segment (mod 8) whose copy did not land
+  int fail_at = 0;  // segment whose copy did not land
   bool ok = true;
   fill(cur);
   fill(nxt);
@@ -206,15 +208,15 @@ __global__ void __launch_bounds__(256, 3) prefix_kernel(XParams p) {
   while (cur.cnt > 0 && ok) {
     const int cnt = cur.cnt;
     const uint32_t multi = __ballot_sync(0xffffffffu, lane < cnt && cur.kb > 1);
-    for (int r0 = 0; r0 < cnt; r0 += 8) {
-      float s[8];
+    for (int r0 = 0; r0 < cnt; r0 += kXRow) {
+      float s[kXRow];
 #pragma unroll
-      for (int r = 0; r < 8; ++r) {
+      for (int r = 0; r < kXRow; ++r) {
         const int i = r0 + r;
         s[r] = 0.f;
         if (i < cnt && ok) {
-          const ST *xp = ring.take(r % kXNB, (uint32_t)(r / kXNB) & 1u, K + __shfl_sync(0xffffffffu, cur.off, i), &ok) + lane;
-          if (!ok) fail_at = r;
+          const ST *xp = ring.take(r % kXNB, (uint32_t)(i / kXNB) & 1u, K + __shfl_sync(0xffffffffu, cur.off, i), &ok) + lane;
+          if (!ok) fail_at = i;
           float x[kXC];
           if (count == kXT) {
 #pragma unroll
@@ -247,9 +249,10 @@ __global__ void __launch_bounds__(256, 3) prefix_kernel(XParams p) {
           s[r] = s2.x + s2.y;
         }
       }
-      const float v = warp_scatter8(s, lane);
-      const int j = r0 + (lane >> 2), at = __shfl_sync(0xffffffffu, cur.idx, j & 31);
-      if ((lane & 3) == 0 && j < cnt) tp[at] = v;
+      const float v = warp_scatter(s, lane);
+      constexpr int kLanes = 32 / kXRow;
+      const int j = r0 + lane / kLanes, at = __shfl_sync(0xffffffffu, cur.idx, j & 31);
+      if (lane % kLanes == 0 && j < cnt) tp[at] = v;
     }
     cur = nxt;
     fill(nxt);

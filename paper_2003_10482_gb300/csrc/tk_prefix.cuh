@@ -100,20 +100,23 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
   return d;
 }
 
-// Sum of the 8 values of every lane over the warp: lane l ends with value l >> 2's
-__device__ __forceinline__ float warp_scatter8(float (&v)[8], int lane) {
+// Sum of the V = 8 or 4 values of every lane over the warp: lane l ends with value
+// l / (32 / V)'s
+template <int V>
+__device__ __forceinline__ float warp_scatter(float (&v)[V], int lane) {
 #pragma unroll
-  for (int k = 16, cnt = 4; cnt >= 1; k >>= 1, cnt >>= 1) {
+  for (int k = 16, cnt = V / 2; cnt >= 1; k >>= 1, cnt >>= 1) {
     const bool up = (lane & k) != 0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < V / 2; ++j) {
       if (j < cnt) {
         const float send = up ? v[j] : v[j + cnt], keep = up ? v[j + cnt] : v[j];
         v[j] = keep + __shfl_xor_sync(0xffffffffu, send, k);
       }
     }
   }
-  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+#pragma unroll
+  for (int k = 16 / V; k >= 2; k >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], k);
   return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
